@@ -57,6 +57,7 @@
 #include <mutex>
 #include <utility>
 
+#include "oz_mode.cuh"
 #include "ozaki_tc.cuh"
 #include "pdl.cuh"
 #include "split_digits.cuh"
@@ -1093,6 +1094,7 @@ struct TcOperator {
   uint16_t *F = nullptr;
   unsigned *eF = nullptr;
   CUtensorMap mK4[4], mF4[4];
+  uint4 *img4[4] = {nullptr, nullptr, nullptr, nullptr};  // modes of the fused product
 };
 
 void free_tc_operator(TcOperator *t) {
@@ -1100,6 +1102,7 @@ void free_tc_operator(TcOperator *t) {
   for (int k = 0; k < 4; ++k) {
     cudaFree(t->K4[k]);
     cudaFree(t->eK4[k]);
+    cudaFree(t->img4[k]);
   }
   cudaFree(t->F);
   cudaFree(t->eF);
@@ -1121,7 +1124,9 @@ cudaError_t ensure_tc_operator_2d(const DevOperator &op, cudaStream_t s) {
   t->So = kOpSlices2;
   t->Sp = kPsiSlices2;
   const int So = t->So, Sp = t->Sp;
-  long long maxw = 0;
+  // modes of up to ozm::kMaxModePoints points take the fused product (oz_mode.cu), which needs
+  // no workspace; maxw, maxM cover the others
+  long long maxw = 0, maxM = 0;
   for (int k = 0; k < 4; ++k) {
     if (op.n[k] < 1 || op.n[k] > kMaxFiber) {
       delete t;
@@ -1133,24 +1138,29 @@ cudaError_t ensure_tc_operator_2d(const DevOperator &op, cudaStream_t s) {
     long long sg = 1;
     for (int j = k + 1; j < 4; ++j) sg *= op.n[j];
     t->sig4[k] = sg;
+    if (op.n[k] <= ozm::kMaxModePoints) continue;
     const long long w = t->M4[k] * t->ld4[k];
     maxw = w > maxw ? w : maxw;
+    maxM = t->M4[k] > maxM ? t->M4[k] : maxM;
   }
   // vectors per chunk: as many as keep the fiber-slice workspace near 1 GB
-  long long ch = (1LL << 30) / (2LL * Sp * maxw);
+  long long ch = maxw ? (1LL << 30) / (2LL * Sp * maxw) : 64;
   t->chunk = (int)(ch < 1 ? 1 : (ch > 64 ? 64 : ch));
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) {
     if (e == cudaSuccess && r != cudaSuccess) e = r;
   };
   for (int k = 0; k < 4; ++k) {
-    chk(cudaMalloc(&t->K4[k], 2LL * So * t->n4[k] * t->ld4[k]));
+    if (t->n4[k] <= ozm::kMaxModePoints)
+      chk(cudaMalloc(&t->img4[k], ozm::image_bytes(t->n4[k])));
+    else
+      chk(cudaMalloc(&t->K4[k], 2LL * So * t->n4[k] * t->ld4[k]));
     chk(cudaMalloc(&t->eK4[k], sizeof(unsigned) * t->n4[k]));
   }
-  long long maxM = 0;
-  for (int k = 0; k < 4; ++k) maxM = t->M4[k] > maxM ? t->M4[k] : maxM;
-  chk(cudaMalloc(&t->F, 2LL * Sp * t->chunk * maxw));
-  chk(cudaMalloc(&t->eF, sizeof(unsigned) * t->chunk * maxM));
+  if (maxw) {
+    chk(cudaMalloc(&t->F, 2LL * Sp * t->chunk * maxw));
+    chk(cudaMalloc(&t->eF, sizeof(unsigned) * t->chunk * maxM));
+  }
   chk(cudaMalloc(&t->err, sizeof(int)));
   if (e != cudaSuccess) {
     free_tc_operator(t);
@@ -1160,6 +1170,10 @@ cudaError_t ensure_tc_operator_2d(const DevOperator &op, cudaStream_t s) {
   bool ok = true;
   for (int k = 0; k < 4; ++k) {
     const int n = t->n4[k];
+    if (t->img4[k]) {
+      ozm::launch_build_image(op.K[k], n, t->img4[k], t->eK4[k], s);
+      continue;
+    }
     chk(cudaMemsetAsync(t->eK4[k], 0, sizeof(unsigned) * n, s));
     launch_exponents(op.K[k], n, n, 0, 1, t->eK4[k], nullptr, s);
     launch_split(op.K[k], n, n, 0, 1, So, t->eK4[k], t->K4[k], t->ld4[k], nullptr, nullptr, 0, s);
@@ -1251,6 +1265,25 @@ cudaError_t launch_apply_h_tc_2d(const DevOperator &op, const double *psi, doubl
     for (int k = 3; k >= 0; --k) {
       const long long M = t.M4[k];
       const int n = t.n4[k];
+      if (t.img4[k]) {
+        ozm::ModeArgs a = {};
+        a.psi = P;
+        a.out = O;
+        a.N = op.N;
+        a.n = n;
+        a.sigma = t.sig4[k];
+        a.image = t.img4[k];
+        a.eK = t.eK4[k];
+        a.nvec = nv;
+        a.store = k == 3;
+        a.V = op.V;
+        a.theta_dev = theta_dev ? theta_dev + v0 : nullptr;
+        a.theta0 = theta;
+        a.err = t.err;
+        const cudaError_t le = ozm::launch_mode_product(a, s);
+        if (le != cudaSuccess) return le;
+        continue;
+      }
       if (t.sig4[k] == 1) {  // the fibers are the rows of the [M][n] view
         long long blocks = (M * nv + 7) / 8;  // 8 rows (warps) per block
         if (blocks > 152LL * 16) blocks = 152LL * 16;

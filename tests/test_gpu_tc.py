@@ -209,3 +209,34 @@ def test_bounded_wait_reports_timeout_and_the_device_stays_usable():
     ctx.device_status()
     assert float(((a - b).norm(dim=1) / (hn * psi.norm(dim=1))).max()) <= 1e-14
     ctx.close()
+
+
+@pytest.mark.parametrize("nx,ny,nvec,offset", [(4, 4, 1, 0), (6, 18, 2, 0), (16, 12, 3, 0),
+                                               (18, 16, 1, 1), (12, 34, 2, 0), (34, 6, 1, 0),
+                                               (8, 48, 2, 0), (8, 50, 1, 0), (6, 64, 2, 0),
+                                               (64, 4, 1, 0), (66, 4, 1, 0), (4, 66, 1, 0),
+                                               (24, 24, 3, 1)])
+def test_apply_h_2d_fused_mode_products(nx, ny, nvec, offset):
+    # the fused mode product at the edges of its 16-point units, where it hands over to the
+    # slice kernels (66 points), for last tiles that are nearly empty, and on vectors that are
+    # only 8-byte aligned.  A fiber is rounded at 2^-55 of its largest entry, K at 2^-62 of its
+    # row's, the results of the four modes once each: each element within 4 (2^-53 + n 2^-55)
+    # of ||H|| max|psi|, well below 1e-14 for n <= 66
+    require_gpu()
+    tps = _tps()
+    n = (nx, nx, ny, ny)
+    L = (8.0,) * 4
+    ctx = make_ctx_2d(20.0, 1.0, n, L, 2.0, 1.0)
+    N, hn = ctx.info()
+    buf = torch.zeros(nvec * N + offset, dtype=torch.float64, device="cuda")
+    psi = buf[offset:].view(nvec, N)
+    psi.copy_(dev(random_normal_block(nvec, N, 11)))
+    psi[-1] *= torch.exp(-torch.linspace(0, 80, N, dtype=torch.float64, device="cuda"))
+    obuf = torch.full((nvec * N + offset,), float("nan"), dtype=torch.float64, device="cuda")
+    out = obuf[offset:].view(nvec, N)
+    ref = torch.empty(nvec, N, dtype=torch.float64, device="cuda")
+    ctx.apply_h(psi, out, -0.3, dtype=tps.F64_TC)
+    ctx.apply_h(psi.clone(), ref, -0.3, dtype=tps.F64)
+    ctx.device_status()
+    assert float(((out - ref).abs().amax(1) / (hn * psi.abs().amax(1))).max()) <= 1e-14
+    ctx.close()
