@@ -4,20 +4,24 @@
 //
 //   out[m][j] (+)= sum_i psi[m][i] K[j][i],   m a fiber of the mode, i, j its points
 //
-// What bounds it: instruction issue.  An element costs about 30 integer and packed FP16
-// instructions to cut into digits and an output about 60 to put together from its eight
-// levels, 0.38 ms per 8-vector apply at 48^4 if every scheduler issued every cycle, against
-// 0.3 ms of tensor time and 0.6 ms for the 24 bytes per element and mode that have to move
-// (psi read, out read and written).  A split kernel that writes the digits to memory and a
-// product kernel that reads them back move 54 bytes.  Measured, 8 vectors at 48^4: 3.62 ms with
-// the two kernels, 1.98 ms with this one.
+// What bounds it: the integer pipe.  An element costs about 35 integer and packed FP16
+// instructions to cut into digits and an output about 45 to put together from its eight
+// levels; the ALU (16 lanes per cycle and scheduler) is 59 % busy, issue 62 %, and the 24 bytes
+// per element and mode that have to move (psi read, out read and written) take 0.62 of the time
+// at the copy rate.  (A split kernel that writes the digits to memory and a product kernel that
+// reads them back move 54 bytes.)  Measured at 48^4 for 3 vectors: 100 us for each of y1, x2 and
+// x1, 115 for y2, 63 for the potential term; a whole apply of 8 vectors 1.18 ms, 3.62 with the
+// split and product kernels.
 //
-// One CTA per SM works through tiles of 128 fibers, every stage of several tiles in flight:
-//   warps 0-7   load psi (two threads per fiber, half of its points each, in registers), take
-//               the fiber's exponent and write the seven digit slices straight into the
-//               operand layout in shared memory (two stages; one for more than 48 points);
-//   warps 8-15  drain the accumulators, recombine the levels and store;
-//   warp 16     issues the MMAs.
+// One CTA per SM works through tiles of 128 fibers, every stage of several tiles in flight
+// (warps for a mode of 33 to 48 points):
+//   warps 0-11   load psi (a warp takes 16 points of 32 fibers, in registers), agree on the
+//                fibers' exponents and write the seven digit slices straight into the operand
+//                layout in shared memory (two stages; one for more than 48 points);
+//   warps 12-27  drain the accumulators, recombine the levels and store;
+//   warp 28      issues the MMAs.
+// (Eight producer and eight epilogue warps, with twice the registers: 115 us per mode instead
+// of 100.)
 // The output columns are taken 16 at a time, eight levels x 16 columns = 128 TMEM columns, so
 // that four of these sub-tiles fit in tensor memory and the epilogue of one runs under the MMAs
 // of the next.  A narrow MMA costs ~45 cycles whatever its width (measured), and a product of
@@ -54,8 +58,6 @@ constexpr int kSA = 7, kSB = 8, kL = 8;  // digits of psi, of K, levels kept (i 
 constexpr int kRows = 128;               // fibers per tile
 constexpr int kCols = 16;                // output columns per sub-tile
 constexpr int kAcc = 4;                  // sub-tiles in tensor memory
-constexpr int kProdWarps = 8, kEpiWarps = 8, kMmaWarp = kProdWarps + kEpiWarps;
-constexpr int kThreads = 32 * (kMmaWarp + 1);
 constexpr int kExpRing = 8;              // tiles whose fiber exponents are kept
 constexpr uint32_t kChunk = kRows * 16;  // bytes of one 16-byte column of K
 constexpr uint32_t kTmemCols = 512;
@@ -68,22 +70,26 @@ struct Cfg {
   static constexpr uint32_t kAStage = kSA * kSlice;
   static constexpr uint32_t kB = KC * kSlice;                  // 8 slices x 16 rows per sub-tile
   static constexpr int kStages = KC <= 3 ? 2 : 1;
-  static constexpr uint32_t kSmem =
-      1024 + kStages * kAStage + kB + kExpRing * kRows * 4 + KC * kCols * 4 + 256;
+  static constexpr int kProdWarps = 4 * KC;           // a unit of 16 points of 32 fibers each
+  static constexpr int kEpiWarps = KC <= 3 ? 16 : 8;  // as many as 1024 threads leave
+  static constexpr int kEpiCols = 4 * kCols / kEpiWarps;  // columns of a sub-tile per warp
+  static constexpr int kMmaWarp = kProdWarps + kEpiWarps;
+  static constexpr int kThreads = 32 * (kMmaWarp + 1);
+  static constexpr uint32_t kSmem = 1024 + kStages * kAStage + kB +
+                                    (kExpRing + 2 * KC) * kRows * 4 + KC * kCols * 4 + 256;
 };
 
 struct Args {
-  const double *psi, *V, *theta_dev;
+  const double *psi;
   double *out;
   long long N;
   unsigned M, n, sigma;
   const uint4 *image;
   const unsigned *eK;
-  double theta0;
   int *err;
   long long tiles;
   unsigned tm;   // tiles per vector
-  int store, vec;  // vec: sigma == 1 and 32-byte accesses are aligned
+  int w1, w9, w17, w25;  // 2, 2^9, 2^17, 2^25 (see level_sum)
 };
 
 // Shared-memory matrix descriptor, K-major, no swizzle: bits 0-13 start address >> 4, bits
@@ -110,19 +116,20 @@ __device__ __forceinline__ void st4(double *p, const double (&v)[4]) {
                : "memory");
 }
 
-// round(x 2^(55 - E)) + 128 (1 + 2^8 + .. + 2^48), E = raw_max - 1022 (|x| < 2^E): bytes 0 .. 5
-// are the lower six digits plus 128, the bits from 48 on the top digit plus 128 (0 .. 256).
-// Subnormals count as zero.
-__device__ __forceinline__ uint64_t biased55(double x, unsigned raw_max) {
+// round(x 2^(55 - E)) + 128 (1 + 2^8 + .. + 2^48), E = raw_max - 1022 (|x| < 2^E), mxe =
+// raw_max << 20: bytes 0 .. 5 are the lower six digits plus 128, the bits from 48 on the top
+// digit plus 128 (0 .. 256).  Subnormals count as zero.
+__device__ __forceinline__ uint64_t biased55(double x, unsigned mxe) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned ex = (hi >> 20) & 0x7FFu;
-  const unsigned sh = ex ? min(raw_max - ex, 63u) : 63u;
-  // the mantissa times 8 (56 bits), shifted right, rounded to nearest (half away from zero)
+  const unsigned exe = hi & 0x7FF00000u;
+  const unsigned sh = exe ? min((mxe - exe) >> 20, 63u) : 63u;
+  // the mantissa times 8 (56 bits), shifted right; with s = 0 or -1 the sign,
+  // (a ^ s) + 2 bias + 1 halved is bias +- round(a / 2), halves away from zero
   const uint64_t m =
       ((uint64_t)((((hi & 0xFFFFFu) | 0x100000u) << 3) | (lo >> 29)) << 32) | (lo << 3);
-  const uint64_t a = ((m >> sh) + 1) >> 1;
-  const uint64_t bias = 0x0080808080808080ULL;
-  return (hi >> 31) ? bias - a : bias + a;
+  const uint64_t a = m >> sh;
+  const uint64_t s = (uint64_t)(long long)((int)hi >> 31);
+  return ((a ^ s) + 0x0101010101010101ULL) >> 1;
 }
 
 // The seven digits of two neighbouring elements as FP16 pairs, most significant first.
@@ -145,17 +152,51 @@ __device__ __forceinline__ void digit_pairs(uint64_t u0, uint64_t u1, uint32_t (
   }
 }
 
+// sum_l d_l 2^(104 - 8 l) 2^(E - 117) rounded to FP64, E the sum of the two exponents.  As
+// sum_i |K[j][i]| < 2^(exponent of row j) the sum is below 2^E, so the levels add up modulo
+// 2^64 to its integer in units of 2^(E - 62); of level 7 (unit 2^(E - 69)) the part below is
+// rounded away, a quarter of what the digit pairs that are not kept weigh (2^(E - 60.5), root
+// mean square at 48 points).  One conversion on the FP64 pipe, otherwise idle here, rounds the
+// integer (a warp instruction takes that pipe ~64 cycles: about one per output is what fits
+// under the integer work; rounding by integer instructions costs ~20 more of them).  The
+// powers of two come from the kernel's arguments: as constants they would become shifts and
+// adds on the ALU, the busiest pipe, where the multiply-adds run on the FMA pipe.
+__device__ __forceinline__ double level_sum(const int (&d)[kL], int E, const Args &g) {
+  const int t7 = (d[7] + 64) >> 7;
+  long long t;
+  asm("{\n\t.reg .b64 t;\n\t"
+      "cvt.s64.s32 t, %5;\n\t"
+      "mad.wide.s32 t, %4, %6, t;\n\t"
+      "mad.wide.s32 t, %3, %7, t;\n\t"
+      "mad.wide.s32 t, %2, %8, t;\n\t"
+      "mad.wide.s32 %0, %1, %9, t;\n\t}"
+      : "=l"(t)
+      : "r"(d[3]), "r"(d[4]), "r"(d[5]), "r"(d[6]), "r"(t7), "r"(g.w1), "r"(g.w9), "r"(g.w17),
+        "r"(g.w25));
+  const unsigned top = (unsigned)(d[0] * g.w17) + (unsigned)(d[1] * g.w9) +
+                       (unsigned)(d[2] * g.w1);
+  t = (long long)((unsigned long long)t + ((unsigned long long)top << 32));
+  const int e = E - 62;
+  if (e < -1000 || e > 900) {  // near the ends of the range: two factors
+    const int h = e / 2;
+    return (double)t * b256::pow2d(h) * b256::pow2d(e - h);
+  }
+  // times 2^e in the exponent field (1023 .. 1086 for a nonzero integer)
+  const double v = (double)t;
+  const int hi = __double2hiint(v);
+  return __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(v));
+}
+
 // The digit image of K (n x n, row-major): for every sub-tile of 16 rows of K, 128 rows (digit
-// j of row c at 16 j + c) x 16 KC points in the operand layout; zeros beyond n.
+// j of row c at 16 j + c) x 16 KC points in the operand layout; zeros beyond n.  A row's
+// exponent is its absolute sum's (see level_sum).
 __global__ void k_build_image(const double *__restrict__ K, int n, int kc,
                               uint4 *__restrict__ image, unsigned *__restrict__ eK) {
   extern __shared__ unsigned ex[];  // exponents of the n rows
   for (int r = threadIdx.x; r < n; r += blockDim.x) {
-    unsigned e = 0;
-    for (int i = 0; i < n; ++i) {
-      const unsigned t = b256::raw_exp(K[(long long)r * n + i]);
-      e = t > e ? t : e;
-    }
+    double sum = 0.0;
+    for (int i = 0; i < n; ++i) sum += fabs(K[(long long)r * n + i]);
+    const unsigned e = b256::raw_exp(sum);
     ex[r] = e;
     if (blockIdx.x == 0) eK[r] = e;
   }
@@ -192,8 +233,14 @@ __global__ void k_build_image(const double *__restrict__ K, int n, int kc,
   }
 }
 
-template <int KC>
-__global__ void __launch_bounds__(kThreads, 1) k_mode_product(const __grid_constant__ Args g) {
+// What the epilogue does with a product: adds it to memory, by an atomic that returns nothing
+// (one term per element and launch, so the sum of the modes is taken in launch order); stores
+// it; stores it, the fibers' points being contiguous and 32-byte accesses aligned.
+enum Epi { kAdd = 0, kStore = 1, kStoreVec = 2 };
+
+template <int KC, Epi EPI>
+__global__ void __launch_bounds__(Cfg<KC>::kThreads, 1)
+k_mode_product(const __grid_constant__ Args g) {
   using C = Cfg<KC>;
   extern __shared__ uint8_t raw_smem[];
   __shared__ int abort_flag;
@@ -201,7 +248,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mode_product(const __grid_const
       (reinterpret_cast<uintptr_t>(raw_smem) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t *sA = base, *sB = base + C::kStages * C::kAStage;
   unsigned *sExp = reinterpret_cast<unsigned *>(sB + C::kB);  // [kExpRing][kRows]
-  int *sEn = reinterpret_cast<int *>(sExp + kExpRing * kRows);
+  unsigned *sMax = sExp + kExpRing * kRows;                   // [2][KC][kRows]
+  int *sEn = reinterpret_cast<int *>(sMax + 2 * KC * kRows);  // [KC * kCols]
   uint64_t *bars = reinterpret_cast<uint64_t *>(sEn + KC * kCols);
   uint64_t *fullA = bars, *emptyA = bars + 2, *accum = bars + 4, *accfree = accum + kAcc;
   uint64_t *drained = accfree + kAcc;
@@ -211,22 +259,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_mode_product(const __grid_const
   if (threadIdx.x == 0) {
     pdl_trigger();
     for (int i = 0; i < 2; ++i) {
-      tc::mbar_init(&fullA[i], kProdWarps);
+      tc::mbar_init(&fullA[i], C::kProdWarps);
       tc::mbar_init(&emptyA[i], 1);
     }
     for (int i = 0; i < kAcc; ++i) {
       tc::mbar_init(&accum[i], 1);
-      tc::mbar_init(&accfree[i], kEpiWarps);
+      tc::mbar_init(&accfree[i], C::kEpiWarps);
     }
     tc::mbar_init(drained, 1);
     abort_flag = 0;
     tc::fence_barrier_init();
   }
-  if (warp == kMmaWarp) tc::tmem_alloc(holder, kTmemCols);
+  if (warp == C::kMmaWarp) tc::tmem_alloc(holder, kTmemCols);
   {
     uint4 *dst = reinterpret_cast<uint4 *>(sB);
-    for (unsigned i = threadIdx.x; i < C::kB / 16; i += kThreads) dst[i] = g.image[i];
-    for (unsigned i = threadIdx.x; i < KC * kCols; i += kThreads)
+    for (unsigned i = threadIdx.x; i < C::kB / 16; i += C::kThreads) dst[i] = g.image[i];
+    for (unsigned i = threadIdx.x; i < KC * kCols; i += C::kThreads)
       sEn[i] = i < g.n ? (int)g.eK[i] - 1022 : 0;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -237,67 +285,119 @@ __global__ void __launch_bounds__(kThreads, 1) k_mode_product(const __grid_const
   // the operator's image above is older than the previous kernel; everything below is not
   pdl_wait();
 
-  if (warp < kProdWarps) {
-    // ---- producers: thread (fiber, half of the points)
-    constexpr int PT = KC * 8;
-    const unsigned fib = warp * 16 + (lane & 15), half = lane >> 4;
-    const unsigned i0 = half * PT;
+  if (warp < C::kProdWarps) {
+    // ---- producers: a warp takes one unit of 16 points of 32 fibers, lane = fiber
+    const unsigned group = warp & 3, unit = warp >> 2;
+    const unsigned i0 = unit * 16;
+    // kAdd: lane = fiber, its 16 points, loads across fibers.  kStoreVec: the unit is 128
+    // contiguous bytes of a fiber; a lane takes a quarter of it of four fibers (lane % 8 + 8 k),
+    // so that a warp's load covers whole lines of 8 fibers
+    constexpr int FL = EPI == kStoreVec ? 4 : 1;  // fibers per lane
+    const unsigned f0 = group * 32 + (EPI == kStoreVec ? lane & 7 : lane);
+    const unsigned piece = EPI == kStoreVec ? lane >> 3 : 0;
     int it = 0;
     for (long long t = blockIdx.x; t < g.tiles; t += gridDim.x, ++it) {
       const unsigned v = (unsigned)(t / g.tm), r = (unsigned)(t - (long long)v * g.tm);
-      const unsigned m = r * kRows + fib;
-      const bool valid = m < g.M;
-      const double *p = g.psi + (long long)v * g.N +
-                        (valid ? (long long)(m / g.sigma) * ((long long)g.n * g.sigma) +
-                                     m % g.sigma
-                               : 0);
-      double x[PT];
-      if (g.vec) {  // contiguous fibers of a multiple of four points
+      double x[16];
+      unsigned mx[FL];
+      if constexpr (EPI == kStoreVec) {  // a multiple of four points
+        const unsigned i = i0 + piece * 4;
 #pragma unroll
-        for (int e = 0; e < PT; e += 4) {
+        for (int k = 0; k < 4; ++k) {
+          const unsigned m = r * kRows + f0 + 8 * k;
           double w[4] = {0.0, 0.0, 0.0, 0.0};
-          if (valid && i0 + e < g.n) ld4(p + i0 + e, w);
+          if (m < g.M && i < g.n) ld4(g.psi + (long long)v * g.N + (long long)m * g.n + i, w);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) x[e + k] = w[k];
+          for (int e = 0; e < 4; ++e) x[4 * k + e] = w[e];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          unsigned e = 0;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            e = max(e, (unsigned)__double2hiint(x[4 * k + j]) & 0x7FF00000u);
+          e = max(e, __shfl_xor_sync(0xffffffffu, e, 8));
+          mx[k] = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
+        }
+      } else {
+        const unsigned m = r * kRows + f0;
+        const bool valid = m < g.M;
+        const double *p = g.psi + (long long)v * g.N + (long long)i0 * g.sigma;
+        if (valid) p += (long long)(m / g.sigma) * ((long long)g.n * g.sigma) + m % g.sigma;
+        const int points = valid ? (int)g.n - (int)i0 : 0;  // of this thread
+        unsigned e0 = 0;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          x[e] = e < points ? *p : 0.0;
+          p += g.sigma;
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) e0 = max(e0, (unsigned)__double2hiint(x[e]) & 0x7FF00000u);
+        mx[0] = e0;
+      }
+      if constexpr (KC > 1) {  // the fibers' exponents over their units
+        unsigned *s = sMax + (it & 1) * (KC * kRows) + f0;
+        if (piece == 0)
+#pragma unroll
+          for (int k = 0; k < FL; ++k) s[unit * kRows + 8 * k] = mx[k];
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(32 * KC) : "memory");
+#pragma unroll
+        for (int k = 0; k < FL; ++k)
+#pragma unroll
+          for (int j = 0; j < KC; ++j) mx[k] = max(mx[k], s[j * kRows + 8 * k]);
+      }
+      const int st = it % C::kStages;
+      // after a failure the units of a group still meet at their barrier: all of them go on
+      // to the last tile without waiting or writing
+      bool ok = !__shfl_sync(0xffffffffu, *((volatile int *)&abort_flag), 0);
+      if (ok) ok = tc::mbar_wait(&emptyA[st], ((it / C::kStages) & 1) ^ 1, g.err, 2);
+      if (!__all_sync(0xffffffffu, ok)) {
+        atomicExch(&abort_flag, 1);
+        continue;
+      }
+      if (unit == 0 && piece == 0)
+#pragma unroll
+        for (int k = 0; k < FL; ++k) sExp[(it % kExpRing) * kRows + f0 + 8 * k] = mx[k] >> 20;
+      uint8_t *dst = sA + st * C::kAStage + (unit * 2) * kChunk + f0 * 16;
+      if constexpr (EPI == kStoreVec) {
+        dst += (piece >> 1) * kChunk + (piece & 1) * 8;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          uint32_t d[2][kSA];
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            digit_pairs(biased55(x[4 * k + 2 * j], mx[k]), biased55(x[4 * k + 2 * j + 1], mx[k]),
+                        d[j]);
+#pragma unroll
+          for (int i = 0; i < kSA; ++i)
+            *reinterpret_cast<uint2 *>(dst + i * C::kSlice + 8 * k * 16) =
+                make_uint2(d[0][i], d[1][i]);
         }
       } else {
 #pragma unroll
-        for (int e = 0; e < PT; ++e)
-          x[e] = valid && i0 + e < g.n ? p[(long long)(i0 + e) * g.sigma] : 0.0;
-      }
-      unsigned mx = 0;
+        for (int c = 0; c < 2; ++c) {
+          uint32_t d[4][kSA];
 #pragma unroll
-      for (int e = 0; e < PT; ++e) mx = max(mx, (unsigned)__double2hiint(x[e]) & 0x7FF00000u);
-      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16)) >> 20;
-      const int st = it % C::kStages;
-      bool ok = tc::mbar_wait(&emptyA[st], ((it / C::kStages) & 1) ^ 1, g.err, 2);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok || *((volatile int *)&abort_flag)) {
-        atomicExch(&abort_flag, 1);
-        break;
-      }
-      if (half == 0) sExp[(it % kExpRing) * kRows + fib] = mx;
-      uint8_t *dst = sA + st * C::kAStage + (half * KC) * kChunk + fib * 16;
+          for (int k = 0; k < 4; ++k)
+            digit_pairs(biased55(x[c * 8 + 2 * k], mx[0]), biased55(x[c * 8 + 2 * k + 1], mx[0]),
+                        d[k]);
 #pragma unroll
-      for (int c = 0; c < KC; ++c) {
-        uint32_t d[4][kSA];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          digit_pairs(biased55(x[c * 8 + 2 * k], mx), biased55(x[c * 8 + 2 * k + 1], mx), d[k]);
-#pragma unroll
-        for (int i = 0; i < kSA; ++i)
-          *reinterpret_cast<uint4 *>(dst + i * C::kSlice + c * kChunk) =
-              make_uint4(d[0][i], d[1][i], d[2][i], d[3][i]);
+          for (int i = 0; i < kSA; ++i)
+            *reinterpret_cast<uint4 *>(dst + i * C::kSlice + c * kChunk) =
+                make_uint4(d[0][i], d[1][i], d[2][i], d[3][i]);
+        }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&fullA[st]);
     }
-  } else if (warp < kMmaWarp) {
-    // ---- epilogue: TMEM lanes 32 (warp % 4) .. + 31 (fibers), 8 of a sub-tile's 16 columns
-    const int quarter = warp & 3, half = (warp - kProdWarps) >> 2;
+  } else if (warp < C::kMmaWarp) {
+    // ---- epilogue: TMEM lanes 32 (warp % 4) .. + 31 (fibers), kEpiCols columns of a sub-tile
+    constexpr int EC = C::kEpiCols;
+    static_assert(C::kProdWarps % 4 == 0 && EC % 4 == 0, "");
+    const int quarter = warp & 3, part = (warp - C::kProdWarps) >> 2;
     const unsigned row = 32 * quarter + lane;
-    const uint32_t trow = tmem + ((uint32_t)(32 * quarter) << 16) + half * 8;
+    const uint32_t trow = tmem + ((uint32_t)(32 * quarter) << 16) + part * EC;
     int it = 0;
     unsigned u = 0;  // sub-tile counter
     bool alive = true;
@@ -311,6 +411,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mode_product(const __grid_const
       double *o = g.out + (long long)v * g.N + mb;
       for (int s = 0; s < KC; ++s, ++u) {
         const unsigned st = u % kAcc;
+        const unsigned c0 = s * kCols + part * EC;
         bool ok = tc::mbar_wait(&accum[st], (u / kAcc) & 1, g.err, 5);
         ok = __all_sync(0xffffffffu, ok);
         const int aborted = __shfl_sync(0xffffffffu, *((volatile int *)&abort_flag), 0);
@@ -320,62 +421,42 @@ __global__ void __launch_bounds__(kThreads, 1) k_mode_product(const __grid_const
         }
         tc::tc_fence_after();
         const int Em = (int)sExp[(it % kExpRing) * kRows + row] - 1022;
-        double val[8];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < EC; h += 4) {
           uint32_t rr[kL][4];
 #pragma unroll
           for (int l = 0; l < kL; ++l)
-            tc::tmem_ld_x4(trow + st * (kL * kCols) + l * kCols + h * 4, rr[l]);
+            tc::tmem_ld_x4(trow + st * (kL * kCols) + l * kCols + h, rr[l]);
           tc::tmem_ld_wait();
-          if (h == 1) {  // the accumulators are read: the MMAs may overwrite them
+          if (h + 4 == EC) {  // the accumulators are read: the MMAs may overwrite them
             tc::tc_fence_before();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&accfree[st]);
           }
+          double val[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             int d[kL];
 #pragma unroll
             for (int l = 0; l < kL; ++l) d[l] = __float2int_rn(__uint_as_float(rr[l][q]));
-            const long long hi = (((long long)d[0] * 256 + d[1]) * 256 + d[2]) * 256 + d[3];
-            const long long lo = (((long long)d[4] * 256 + d[5]) * 256 + d[6]) * 256 + d[7];
-            val[h * 4 + q] =
-                b256::combine(hi, lo, Em + sEn[s * kCols + half * 8 + h * 4 + q] + 1);
+            val[q] = level_sum(d, Em + sEn[c0 + h + q], g);
           }
-        }
-        const unsigned c0 = s * kCols + half * 8;
-        if (!valid) continue;
-        if (g.store) {
-          const double th = g.theta_dev ? g.theta_dev[v] : g.theta0;
-          const double *pp = g.psi + (long long)v * g.N + mb, *vp = g.V + mb;
-          if (g.vec) {
+          const unsigned c = c0 + h;
+          if (valid) {
+            if constexpr (EPI == kStoreVec) {
+              if (c < g.n) st4(o + c, val);
+            } else {
+              double *oc = o + (long long)c * g.sigma;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const unsigned c = c0 + 4 * h;
-              if (c < g.n) {
-                double a[4], b[4], w[4];
-                ld4(vp + c, a);
-                ld4(pp + c, b);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) w[q] = fma(a[q] - th, b[q], val[h * 4 + q]);
-                st4(o + c, w);
-              }
+              for (int q = 0; q < 4; ++q, oc += g.sigma)
+                if (c + q < g.n) {
+                  if constexpr (EPI == kStore)
+                    *oc = val[q];
+                  else
+                    atomicAdd(oc, val[q]);
+                }
             }
-          } else {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              if (c0 + q < g.n) {
-                const long long i = (long long)(c0 + q) * g.sigma;
-                o[i] = fma(vp[i] - th, pp[i], val[q]);
-              }
           }
-        } else {
-          // each element belongs to one thread of one CTA per launch: the sum of the modes
-          // is taken in launch order
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (c0 + q < g.n) atomicAdd(o + (long long)(c0 + q) * g.sigma, val[q]);
         }
       }
     }
@@ -420,23 +501,83 @@ __global__ void __launch_bounds__(kThreads, 1) k_mode_product(const __grid_const
   __syncwarp();
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == kMmaWarp) tc::tmem_dealloc(tmem, kTmemCols);
+  if (warp == C::kMmaWarp) tc::tmem_dealloc(tmem, kTmemCols);
 }
 
-template <int KC>
+// out += (V - theta) psi.  Bound by memory: V is read once for all vectors, psi and out read,
+// out written, two unknowns per thread where 16-byte accesses are aligned.  (In a mode
+// product's epilogue, whose loads of V and psi wait for memory in line with the products, the
+// term cost 83 us for 3 vectors at 48^4, here 63.)
+template <int W>
+__global__ void __launch_bounds__(256)
+k_potential_term(const double *__restrict__ psi, const double *__restrict__ V,
+                 double *out, long long N, int nvec,
+                 const double *__restrict__ theta_dev, double theta0) {
+  if (threadIdx.x == 0) pdl_trigger();
+  pdl_wait();
+  const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * W;
+  if (i >= N) return;
+  double w[W], x[4][W], y[4][W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) w[k] = V[i + k];
+  if (!theta_dev)
+#pragma unroll
+    for (int k = 0; k < W; ++k) w[k] -= theta0;
+  for (int v0 = 0; v0 < nvec; v0 += 4) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      if (v0 + v < nvec) {
+        const long long j = (long long)(v0 + v) * N + i;
+        if constexpr (W == 2) {
+          const double2 a = *reinterpret_cast<const double2 *>(psi + j);
+          const double2 b = *reinterpret_cast<const double2 *>(out + j);
+          x[v][0] = a.x;
+          x[v][1] = a.y;
+          y[v][0] = b.x;
+          y[v][1] = b.y;
+        } else {
+          x[v][0] = psi[j];
+          y[v][0] = out[j];
+        }
+      }
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      if (v0 + v < nvec) {
+        double *o = out + (long long)(v0 + v) * N + i;
+        const double th = theta_dev ? theta_dev[v0 + v] : 0.0;
+#pragma unroll
+        for (int k = 0; k < W; ++k) y[v][k] = fma(theta_dev ? w[k] - th : w[k], x[v][k], y[v][k]);
+        if constexpr (W == 2)
+          *reinterpret_cast<double2 *>(o) = make_double2(y[v][0], y[v][1]);
+        else
+          *o = y[v][0];
+      }
+  }
+}
+
+template <int KC, Epi EPI>
 cudaError_t launch_kc(const Args &g, cudaStream_t s) {
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_mode_product<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    attr = cudaFuncSetAttribute(k_mode_product<KC, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)Cfg<KC>::kSmem);
   });
   if (attr != cudaSuccess) return attr;
   const unsigned grid = (unsigned)(g.tiles < 152 ? g.tiles : 152);
   count_launch();
-  const cudaError_t e = launch_pdl(k_mode_product<KC>, dim3(grid), dim3(kThreads),
+  const cudaError_t e = launch_pdl(k_mode_product<KC, EPI>, dim3(grid), dim3(Cfg<KC>::kThreads),
                                    Cfg<KC>::kSmem, s, g);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <int KC>
+cudaError_t launch_epi(const Args &g, Epi epi, cudaStream_t s) {
+  switch (epi) {
+    case kStore: return launch_kc<KC, kStore>(g, s);
+    case kStoreVec: return launch_kc<KC, kStoreVec>(g, s);
+    default: return launch_kc<KC, kAdd>(g, s);
+  }
 }
 
 int units(int n) { return (n + 15) / 16; }
@@ -453,14 +594,27 @@ void launch_build_image(const double *K, int n, uint4 *image, unsigned *eK, cuda
   k_build_image<<<16, 256, n * sizeof(unsigned), s>>>(K, n, units(n), image, eK);
 }
 
+cudaError_t launch_potential_term(const double *psi, const double *V, double *out, long long N,
+                                  int nvec, const double *theta_dev, double theta0,
+                                  cudaStream_t s) {
+  const uintptr_t al = reinterpret_cast<uintptr_t>(psi) | reinterpret_cast<uintptr_t>(out) |
+                       reinterpret_cast<uintptr_t>(V);
+  const bool two = N % 2 == 0 && (al & 15) == 0;
+  const long long blocks = (N / (two ? 2 : 1) + 255) / 256;
+  if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
+  count_launch();
+  const cudaError_t e =
+      launch_pdl(two ? k_potential_term<2> : k_potential_term<1>, dim3((unsigned)blocks),
+                 dim3(256), 0, s, psi, V, out, N, nvec, theta_dev, theta0);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 cudaError_t launch_mode_product(const ModeArgs &a, cudaStream_t s) {
   if (a.n < 1 || a.n > kMaxModePoints || a.nvec < 1) return cudaErrorInvalidValue;
   const long long M = a.N / a.n;
   if (M > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
   Args g = {};
   g.psi = a.psi;
-  g.V = a.V;
-  g.theta_dev = a.theta_dev;
   g.out = a.out;
   g.N = a.N;
   g.M = (unsigned)M;
@@ -468,19 +622,21 @@ cudaError_t launch_mode_product(const ModeArgs &a, cudaStream_t s) {
   g.sigma = (unsigned)a.sigma;
   g.image = a.image;
   g.eK = a.eK;
-  g.theta0 = a.theta0;
   g.err = a.err;
   g.tm = (unsigned)((M + kRows - 1) / kRows);
   g.tiles = (long long)g.tm * a.nvec;
-  g.store = a.store ? 1 : 0;
-  const uintptr_t al = reinterpret_cast<uintptr_t>(a.psi) | reinterpret_cast<uintptr_t>(a.out) |
-                       reinterpret_cast<uintptr_t>(a.V);
-  g.vec = a.sigma == 1 && a.n % 4 == 0 && (al & 31) == 0;
+  g.w1 = 1 << 1;
+  g.w9 = 1 << 9;
+  g.w17 = 1 << 17;
+  g.w25 = 1 << 25;
+  const uintptr_t al = reinterpret_cast<uintptr_t>(a.psi) | reinterpret_cast<uintptr_t>(a.out);
+  const bool vec = a.sigma == 1 && a.n % 4 == 0 && (al & 31) == 0;
+  const Epi epi = !a.store ? kAdd : vec ? kStoreVec : kStore;
   switch (units(a.n)) {
-    case 1: return launch_kc<1>(g, s);
-    case 2: return launch_kc<2>(g, s);
-    case 3: return launch_kc<3>(g, s);
-    default: return launch_kc<4>(g, s);
+    case 1: return launch_epi<1>(g, epi, s);
+    case 2: return launch_epi<2>(g, epi, s);
+    case 3: return launch_epi<3>(g, epi, s);
+    default: return launch_epi<4>(g, epi, s);
   }
 }
 

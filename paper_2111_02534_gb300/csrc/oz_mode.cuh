@@ -27,13 +27,15 @@ struct ModeArgs {
   const uint4 *image;       // launch_build_image
   const unsigned *eK;
   int nvec;
-  bool store;               // true: out = K psi + (V - theta) psi, else out += K psi
-  const double *V;          // [N] (store)
-  const double *theta_dev;  // theta of each vector (null: theta0)
-  double theta0;
+  bool store;               // true: out = K psi, else out += K psi
   int *err;                 // device flag of timed-out waits
 };
+// One mode's product.
 cudaError_t launch_mode_product(const ModeArgs &a, cudaStream_t s);
+// out += (V - theta) psi; theta_dev: theta of each vector (null: theta0).
+cudaError_t launch_potential_term(const double *psi, const double *V, double *out, long long N,
+                                  int nvec, const double *theta_dev, double theta0,
+                                  cudaStream_t s);
 
 }  // namespace ozm
 }  // namespace tps

@@ -43,11 +43,11 @@
 // is order-independent).  Operand tiles reach shared memory by TMA (128-byte swizzle,
 // K-major), one thread issues tcgen05.mma into tensor memory, and eight warps drain it.
 //
-// The 2D H-apply (Eq. tensor_op2D) runs its four mode products one after the other, each
-// over the fibers of its mode (A = fiber slices, B = K_k slices), with a persistent kernel:
-// one CTA per SM takes tile after tile, its producer, MMA and epilogue warps working on
-// successive tiles at once (the 48-point contraction gives short MMA loops, so a CTA per
-// tile spent most of its time in the epilogue with the tensor pipe idle).
+// The 2D H-apply (Eq. tensor_op2D) runs its four mode products one after the other, modes of
+// up to 64 points by one fused kernel each (oz_mode.cu).  Longer ones, whose digits of 128
+// fibers do not fit in shared memory beside the mode matrix's, take the kernels here: the
+// fibers' digit slices go to memory, and a persistent product kernel (one CTA per SM, its
+// producer, MMA and epilogue warps working on successive tiles at once) multiplies them.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -845,9 +845,6 @@ k_oz_gemm1p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   const int tm = (g.M + kBM - 1) / kBM, tn = (g.N + kBN - 1) / kBN;
   const long long T = (long long)tm * tn * g.nvec;
   const int KB = (g.K + kBK - 1) / kBK;
-  // one K block and one column tile (modes of at most 48 points): every tile multiplies by
-  // the same B slices, loaded once into stage 0 and kept
-  const bool b_fixed = KB == 1 && tn == 1;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kAStages; ++i) {
@@ -883,19 +880,17 @@ k_oz_gemm1p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const int v = (int)(t / ((long long)tm * tn)), r = (int)(t % ((long long)tm * tn));
         const int m0 = (r % tm) * kBM, n0 = (r / tm) * kBN;
         for (int kb = 0; kb < KB && ok; ++kb, ++bcount) {
-          const int sb = b_fixed ? 0 : (int)(bcount % kBStages);
-          const uint32_t rb = b_fixed ? 0u : (uint32_t)(bcount / kBStages);
-          if (!b_fixed || t == blockIdx.x) {
-            if (!tc::mbar_wait(&emptyB[sb], (rb & 1u) ^ 1u, g.err, 1)) {
-              ok = false;
-              break;
-            }
-            tc::mbar_arrive_expect_tx(&fullB[sb], bstage);
-            for (int j = 0; j < SB; ++j)
-              tc::tma_load_3d(sB + sb * bstage + j * b_slice_bytes(), &tmB, &fullB[sb],
-                              kb * kBK, n0, v * g.zB + j);
-            lastB[sb] = (int)(rb & 1u);
+          const int sb = (int)(bcount % kBStages);
+          const uint32_t rb = (uint32_t)(bcount / kBStages);
+          if (!tc::mbar_wait(&emptyB[sb], (rb & 1u) ^ 1u, g.err, 1)) {
+            ok = false;
+            break;
           }
+          tc::mbar_arrive_expect_tx(&fullB[sb], bstage);
+          for (int j = 0; j < SB; ++j)
+            tc::tma_load_3d(sB + sb * bstage + j * b_slice_bytes(), &tmB, &fullB[sb],
+                            kb * kBK, n0, v * g.zB + j);
+          lastB[sb] = (int)(rb & 1u);
           for (int i = 0; i < SA; ++i, ++acount) {
             const int sa = (int)(acount % kAStages);
             const uint32_t ra = (uint32_t)(acount / kAStages);
@@ -935,8 +930,8 @@ k_oz_gemm1p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
         tc::tc_fence_after();
         for (int kb = 0; kb < KB && ok; ++kb, ++bcount) {
-          const int sb = b_fixed ? 0 : (int)(bcount % kBStages);
-          const uint32_t rb = b_fixed ? 0u : (uint32_t)(bcount / kBStages);
+          const int sb = (int)(bcount % kBStages);
+          const uint32_t rb = (uint32_t)(bcount / kBStages);
           if (!tc::mbar_wait(&fullB[sb], rb & 1u, g.err, 3)) {
             ok = false;
             break;
@@ -967,7 +962,7 @@ k_oz_gemm1p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
             tc::mma_commit(&emptyA[sa]);  // the A stage is free once these MMAs are done
           }
-          if (ok && !b_fixed) tc::mma_commit(&emptyB[sb]);
+          if (ok) tc::mma_commit(&emptyB[sb]);
         }
         // the tile's accumulators are complete once its MMAs are (after a failure: only so
         // that nothing is in flight at exit)
@@ -1262,6 +1257,9 @@ cudaError_t launch_apply_h_tc_2d(const DevOperator &op, const double *psi, doubl
     const int nv = nvec - v0 < t.chunk ? nvec - v0 : t.chunk;
     const double *P = psi + (long long)v0 * op.N;
     double *O = out + (long long)v0 * op.N;
+    // y2 stores, with the potential term unless it is a fused product (whose form for
+    // contiguous fibers only stores: reading what it adds to cost 40 us for 3 vectors at 48^4);
+    // the other modes add, coalesced
     for (int k = 3; k >= 0; --k) {
       const long long M = t.M4[k];
       const int n = t.n4[k];
@@ -1276,9 +1274,6 @@ cudaError_t launch_apply_h_tc_2d(const DevOperator &op, const double *psi, doubl
         a.eK = t.eK4[k];
         a.nvec = nv;
         a.store = k == 3;
-        a.V = op.V;
-        a.theta_dev = theta_dev ? theta_dev + v0 : nullptr;
-        a.theta0 = theta;
         a.err = t.err;
         const cudaError_t le = ozm::launch_mode_product(a, s);
         if (le != cudaSuccess) return le;
@@ -1327,6 +1322,11 @@ cudaError_t launch_apply_h_tc_2d(const DevOperator &op, const double *psi, doubl
       const unsigned grid = (unsigned)(tiles < 152 ? tiles : 152);
       k_oz_gemm1p<<<grid, kPThreads, ozp_smem_bytes(), s>>>(t.mF4[k], t.mK4[k], g);
       const cudaError_t le = cudaGetLastError();
+      if (le != cudaSuccess) return le;
+    }
+    if (t.img4[3]) {
+      const cudaError_t le = ozm::launch_potential_term(
+          P, op.V, O, op.N, nv, theta_dev ? theta_dev + v0 : nullptr, theta, s);
       if (le != cudaSuccess) return le;
     }
   }
