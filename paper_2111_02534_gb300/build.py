@@ -20,7 +20,7 @@ BUILD_DIR = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["gemm_f64.cu", "gemm_f32.cu", "blocks_f64.cu", "jd_kernels.cu", "api.cpp", "jd.cpp",
            "batch.cpp", "gram_noalloc.cu", "ozaki_tc.cu", "mlp.cu", "rr_eigh.cu", "tf32_tc.cu", "update_mma.cu", "host_eig.cpp",
-           "gram_mma.cu", "oz_mode.cu"]
+           "gram_mma.cu", "oz_mode.cu", "oz_fold.cu"]
 
 
 def _nvcc() -> str:

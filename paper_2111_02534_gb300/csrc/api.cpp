@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <limits>
 #include <new>
@@ -46,8 +47,12 @@ std::vector<double> d2_matrix(int n, double L) {
       if (i == j) {
         v = -kPi * kPi / (3.0 * h * h) - 1.0 / 6.0;
       } else {
-        const double s = std::sin((i - j) * h / 2.0);
-        const double sgn = ((i - j) % 2 == 0) ? 1.0 : -1.0;
+        // by the periodic distance, at most n/2: the matrix is then circulant to the last bit
+        // (the tensor-core products use that), and near |i - j| = n the sine is not taken of an
+        // argument near pi, whose rounding it magnifies n-fold
+        const int d = std::min(std::abs(i - j), n - std::abs(i - j));
+        const double s = std::sin(d * h / 2.0);
+        const double sgn = d % 2 == 0 ? 1.0 : -1.0;
         v = -sgn / (2.0 * s * s);
       }
       D[(size_t)i * n + j] = v * scale;
@@ -87,6 +92,7 @@ std::vector<double> transpose(const std::vector<double> &A, int n) {
 
 struct HostMode {
   int n = 0;
+  int symmetry = kModeGeneral;
   std::vector<double> K, S, lam;
   std::vector<double> Sinv;  // S^-1 when the eigenbasis is not orthogonal (else empty)
 };
@@ -95,6 +101,7 @@ struct HostMode {
 HostMode full_mode(int n, double L, double a) {
   HostMode m;
   m.n = n;
+  m.symmetry = kModeCirculant;
   m.K = d2_matrix(n, L);
   for (auto &v : m.K) v *= a;
   std::vector<int> kcol;
@@ -118,6 +125,7 @@ HostMode sector_mode(const HostMode &full, int parity, double L, double a) {
   const int nr = even ? n / 2 + 1 : n / 2 - 1;
   const int off = even ? 0 : 1;
   m.n = nr;
+  m.symmetry = kModeMirror;  // the shift by L maps a sector to itself
   m.K.assign((size_t)nr * nr, 0.0);
   m.S.assign((size_t)nr * nr, 0.0);
   m.lam.assign(nr, 0.0);
@@ -175,6 +183,7 @@ int build_operator(tps_ctx *ctx, DevOperator &op, const std::vector<HostMode> &m
   for (int k = 0; k < op.nmodes; ++k) {
     const HostMode &m = modes[k];
     op.n[k] = m.n;
+    op.symmetry[k] = m.symmetry;
     op.N *= m.n;
     int st;
     if ((st = upload(ctx, &op.K[k], m.K))) return st;

@@ -21,6 +21,10 @@ inline void count_launch() { g_kernel_launches.fetch_add(1, std::memory_order_re
 extern std::atomic<int> g_autotune;
 inline bool autotune_enabled() { return g_autotune.load(std::memory_order_relaxed) != 0; }
 
+// Symmetry of a mode matrix K: none used; circulant and symmetric (a periodic Fourier grid);
+// symmetric under the reversal of the points in both indices (a heavy-exchange sector of one).
+enum { kModeGeneral = 0, kModeCirculant = 1, kModeMirror = 2 };
+
 // ---------------------------------------------------------------------------
 // A discretised Kronecker-sum operator resident on the device:
 //   H = sum_k (I x .. x K_k x .. x I) + diag(V),  K_k = a_k D2_k (dense n_k x n_k),
@@ -32,6 +36,7 @@ inline bool autotune_enabled() { return g_autotune.load(std::memory_order_relaxe
 struct DevOperator {
   int nmodes = 0;
   int n[4] = {0, 0, 0, 0};
+  int symmetry[4] = {0, 0, 0, 0};  // kModeGeneral, ..
   long long N = 0;
   double *K[4] = {nullptr, nullptr, nullptr, nullptr};   // row-major n x n
   double *KT[4] = {nullptr, nullptr, nullptr, nullptr};  // K^T (equal to K for symmetric D2)

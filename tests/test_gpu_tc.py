@@ -240,3 +240,55 @@ def test_apply_h_2d_fused_mode_products(nx, ny, nvec, offset):
     ctx.device_status()
     assert float(((out - ref).abs().amax(1) / (hn * psi.abs().amax(1))).max()) <= 1e-14
     ctx.close()
+
+
+@pytest.mark.parametrize("nx,ny,nvec,offset", [(4, 4, 1, 0), (6, 8, 2, 0), (12, 10, 3, 1),
+                                               (16, 62, 2, 0), (64, 66, 5, 0), (60, 130, 1, 1),
+                                               (146, 34, 2, 0), (128, 256, 3, 0),
+                                               (258, 20, 2, 0), (290, 12, 1, 0),
+                                               (292, 8, 1, 0), (8, 294, 1, 0), (20, 512, 2, 0),
+                                               (580, 16, 1, 0), (16, 584, 1, 0)])
+def test_apply_h_1d_folded(nx, ny, nvec, offset):
+    # the folded H-apply at the edges of its tiles (16 and 64 points, 128 lines) and of the
+    # sizes it takes (146 points a block: 290 and 580 points; 294 and 584 take the dense
+    # products).  Lines are rounded at 2^-61 of their largest entry and the two products once
+    # each; the FMA path's own rounding, n 2^-53 of a row's sum at most, is what the bound covers
+    require_gpu()
+    tps = _tps()
+    ctx = make_ctx_1d(20.0, 1.0, (nx, ny), (20.0, 15.0), 1.0, 1.0)
+    N, hn = ctx.info()
+    buf = torch.zeros(nvec * N + offset, dtype=torch.float64, device="cuda")
+    psi = buf[offset:].view(nvec, N)
+    psi.copy_(dev(random_normal_block(nvec, N, 13)))
+    psi[-1] *= torch.exp(-torch.linspace(0, 60, N, dtype=torch.float64, device="cuda"))
+    obuf = torch.full((nvec * N + offset,), float("nan"), dtype=torch.float64, device="cuda")
+    out = obuf[offset:].view(nvec, N)
+    ref = torch.empty(nvec, N, dtype=torch.float64, device="cuda")
+    ctx.apply_h(psi, out, 0.7, dtype=tps.F64_TC)
+    ctx.apply_h(psi.clone(), ref, 0.7, dtype=tps.F64)
+    ctx.device_status()
+    assert float(((out - ref).abs().amax(1) / (hn * psi.abs().amax(1))).max()) <= 1e-14
+    again = torch.empty_like(out)
+    ctx.apply_h(psi, again, 0.7, dtype=tps.F64_TC)
+    torch.cuda.synchronize()
+    assert torch.equal(out, again)
+    ctx.close()
+
+
+@pytest.mark.parametrize("n,parity", [((64, 48), 1), ((64, 48), 2), ((66, 50), 1), ((62, 64), 2),
+                                      ((130, 36), 1)])
+def test_solve_in_a_sector_with_folded_products(n, parity):
+    # sectors of 33, 31, 34, 30 and 66 points: odd and even reversals
+    require_gpu()
+    tps = _tps()
+    ctx = make_ctx_1d(20.0, 1.0, n, (12.0, 12.0), 2.0, 1.0)
+    ev = torch.empty(3, ctx.info()[0], dtype=torch.float64, device="cuda")
+    lam = []
+    for dt in (tps.F64_TC, tps.F64):
+        opts = tps.default_opts()
+        opts.h64_dtype = dt
+        lam.append(ctx.solve(3, parity, 1e-12, 4, ev, opts=opts)[0])
+    # two solves to a residual of 1e-12 ||H||: eigenvalues to the square of it over the gaps,
+    # and the operator's own rounding
+    assert np.max(np.abs(lam[0] - lam[1])) <= 1e-12 * ctx.info()[1]
+    ctx.close()
