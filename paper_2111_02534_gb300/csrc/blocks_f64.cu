@@ -7,6 +7,7 @@
 #include <mutex>
 #include <utility>
 
+#include "fp_convert.cuh"
 #include "pdl.cuh"
 #include "tps_internal.h"
 
@@ -14,6 +15,26 @@ namespace tps {
 namespace {
 
 constexpr int GT = 256;  // threads of the Gram / update kernels
+
+// An FP64 value in the arithmetic T of a kernel and back; INT: by integer instructions.  The
+// hardware conversions run on GB300's FP64 pipe, which takes a warp instruction per ~64 cycles
+// of a scheduler, more than the ~44 in which the memory delivers a warp's 32 values to one.
+template <typename T, bool INT>
+__device__ __forceinline__ T load_as(double x) {
+  if constexpr (INT)
+    return f32_near(x);
+  else
+    return (T)x;
+}
+template <bool INT>
+__device__ __forceinline__ double as_f64(double x) { return x; }
+template <bool INT>
+__device__ __forceinline__ double as_f64(float x) {
+  if constexpr (INT)
+    return f64_of_f32(x);
+  else
+    return (double)x;
+}
 
 // -------------------------------- Gram ---------------------------------------
 // G_s = A_s^T B_s in one launch.  CTA (c, s, pb) sums the BP x BQ block pb over the rows of
@@ -23,7 +44,10 @@ constexpr int GT = 256;  // threads of the Gram / update kernels
 // register tile fits the shape (16 x 1, 8 x 2, 4 x 4 and smaller), so narrow products do
 // not pay for FMAs on padding; trans = 1 stores the transposed block (the launcher swaps
 // the operands when p < q).  T = float: FP32 products and partial sums on the FP64 data
-// (the low-precision variant; the chunk sums are added in FP64).
+// (the low-precision variant; the chunk sums are added in FP64), bound by the conversions on
+// the FP64 pipe: p = 8, 3 systems of 5.3 M rows 274 us (245 of conversions), 426 with a run of
+// rows per CTA, two CTAs per SM and one thread per value adding the chunks; integer conversions
+// (as in k_update) measured slower here at every shape but p = 8 and 10.
 //
 // Warp reduction of V = BP BQ values by recursive halving: at offset o each lane keeps
 // half of its values and adds the other half of its partner's, so a lane spends V - 1 +
@@ -83,24 +107,24 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
   const int i0 = (pb / qb) * BP, j0 = (pb % qb) * BQ;
   const double *As = A + s * bsa;
   const double *Bs = B + s * bsb;
-  const long long rows_per = (nrows + nchunk - 1) / nchunk;
-  const long long r0 = (long long)c * rows_per;
-  const long long r1 = r0 + rows_per < nrows ? r0 + rows_per : nrows;
+  // the chunks' rows are interleaved, so that the CTAs read neighbouring addresses of the
+  // p + q columns at any time and few pages of memory are in use at once
+  const long long step = (long long)nchunk * GT;
   T acc[V];
 #pragma unroll
   for (int k = 0; k < V; ++k) acc[k] = T(0);
   // two rows per iteration: all of their loads are issued before the first FMA waits
-  long long r = r0 + threadIdx.x;
-  for (; r + GT < r1; r += 2 * GT) {
+  long long r = (long long)c * GT + threadIdx.x;
+  for (; r + step < nrows; r += 2 * step) {
     T a[2][BP], b[2][BQ];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
 #pragma unroll
       for (int i = 0; i < BP; ++i)
-        a[h][i] = (i0 + i < p) ? (T)As[(long long)(i0 + i) * lda + r + h * GT] : T(0);
+        a[h][i] = (i0 + i < p) ? (T)As[(long long)(i0 + i) * lda + r + h * step] : T(0);
 #pragma unroll
       for (int j = 0; j < BQ; ++j)
-        b[h][j] = (j0 + j < q) ? (T)Bs[(long long)(j0 + j) * ldb + r + h * GT] : T(0);
+        b[h][j] = (j0 + j < q) ? (T)Bs[(long long)(j0 + j) * ldb + r + h * step] : T(0);
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -109,7 +133,7 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
 #pragma unroll
         for (int j = 0; j < BQ; ++j) acc[i * BQ + j] = fma(a[h][i], b[h][j], acc[i * BQ + j]);
   }
-  if (r < r1) {
+  if (r < nrows) {
     T a[BP], b[BQ];
 #pragma unroll
     for (int i = 0; i < BP; ++i)
@@ -139,20 +163,26 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
   if (threadIdx.x == 0) ticket = atomicAdd(&count[blk], 1u);
   __syncthreads();
   if (ticket != (unsigned)(nchunk - 1)) return;
-  // last CTA of the block: every other chunk's partial sums are in memory
+  // last CTA of the block: every other chunk's partial sums are in memory.  All threads add
+  // them, GT / V per value, then a tree over those (one thread per value walking the chunks
+  // took up to 50 us)
+  __threadfence();
+  __shared__ double tot[GT];
+  constexpr int parts = GT / V;
+  {
+    const double *src = partial + blk * nchunk * V + threadIdx.x % V;
+    double v = 0.0;
+#pragma unroll 4
+    for (int cc = threadIdx.x / V; cc < nchunk; cc += parts) v += __ldcg(src + (long long)cc * V);
+    tot[threadIdx.x] = v;
+  }
+  for (int o = parts / 2; o > 0; o >>= 1) {
+    __syncthreads();
+    if (threadIdx.x < o * V) tot[threadIdx.x] += tot[threadIdx.x + o * V];
+  }
+  __syncthreads();
   if (threadIdx.x < V) {
-    __threadfence();
-    const double *src = partial + blk * nchunk * V + threadIdx.x;
-    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
-    int cc = 0;
-    for (; cc + 4 <= nchunk; cc += 4) {
-      v0 += __ldcg(src + (long long)(cc + 0) * V);
-      v1 += __ldcg(src + (long long)(cc + 1) * V);
-      v2 += __ldcg(src + (long long)(cc + 2) * V);
-      v3 += __ldcg(src + (long long)(cc + 3) * V);
-    }
-    for (; cc < nchunk; ++cc) v0 += __ldcg(src + (long long)cc * V);
-    const double v = (v0 + v1) + (v2 + v3);
+    const double v = tot[threadIdx.x];
     const int i = i0 + threadIdx.x / BQ, j = j0 + threadIdx.x % BQ;
     if (i < p && j < q) {
       if (trans)
@@ -164,8 +194,11 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
   if (threadIdx.x == 0) count[blk] = 0u;  // re-armed for the next call on this stream
 }
 
-int gram_chunks(long long nrows, int batch, int npb) {
-  const long long want = (2LL * 152 + (long long)batch * npb - 1) / ((long long)batch * npb);
+// Chunks of rows per block: two CTAs per SM in all, four for FP32 products, which wait for
+// memory where FP64 ones wait for the FMA pipe; at least 1024 rows each.
+int gram_chunks(long long nrows, int batch, int npb, bool low) {
+  const long long blocks = (long long)batch * npb;
+  const long long want = ((low ? 4 : 2) * 152LL + blocks - 1) / blocks;
   const long long maxc = (nrows + 1023) / 1024;
   long long c = want < maxc ? want : maxc;
   if (c < 1) c = 1;
@@ -180,7 +213,7 @@ int gram_chunks(long long nrows, int batch, int npb) {
 // combination in FP64.  A grid of at most one wave of CTAs strides over the rows, two
 // rows and four columns of A per thread in flight (a CTA per 256 rows spent most of its
 // life loading Y).
-template <typename T, int BQ>
+template <typename T, int BQ, bool INT>
 __global__ void __launch_bounds__(GT)
 k_update(const double *__restrict__ A, long long lda, long long bsa, int p,
          const double *__restrict__ Y, int ldy, long long bsy, int q, double alpha, double beta,
@@ -205,13 +238,24 @@ k_update(const double *__restrict__ A, long long lda, long long bsa, int p,
     T acc0[BQ], acc1[BQ];
 #pragma unroll
     for (int j = 0; j < BQ; ++j) acc0[j] = acc1[j] = T(0);
+    // narrow updates load the old values with the first columns of A
+    constexpr bool kOld = BQ <= 2;
+    double old0[kOld ? BQ : 1], old1[kOld ? BQ : 1];
+    if constexpr (kOld)
+      if (beta != 0.0)
+#pragma unroll
+        for (int j = 0; j < BQ; ++j) {
+          const double *src = Cs + (long long)(j0 + j < q ? j0 + j : 0) * ldc;
+          old0[j] = src[r0];
+          old1[j] = v1 ? src[r1] : 0.0;
+        }
     int i = 0;
     for (; i + 4 <= p; i += 4) {
       T a0[4], a1[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        a0[u] = (T)As[(long long)(i + u) * lda + r0];
-        a1[u] = v1 ? (T)As[(long long)(i + u) * lda + r1] : T(0);
+        a0[u] = load_as<T, INT>(As[(long long)(i + u) * lda + r0]);
+        a1[u] = v1 ? load_as<T, INT>(As[(long long)(i + u) * lda + r1]) : T(0);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -222,8 +266,8 @@ k_update(const double *__restrict__ A, long long lda, long long bsa, int p,
         }
     }
     for (; i < p; ++i) {
-      const T a0 = (T)As[(long long)i * lda + r0];
-      const T a1 = v1 ? (T)As[(long long)i * lda + r1] : T(0);
+      const T a0 = load_as<T, INT>(As[(long long)i * lda + r0]);
+      const T a1 = v1 ? load_as<T, INT>(As[(long long)i * lda + r1]) : T(0);
 #pragma unroll
       for (int j = 0; j < BQ; ++j) {
         acc0[j] = fma(a0, Ys[i][j], acc0[j]);
@@ -234,8 +278,14 @@ k_update(const double *__restrict__ A, long long lda, long long bsa, int p,
     for (int j = 0; j < BQ; ++j) {
       if (j0 + j >= q) break;
       double *dst = Cs + (long long)(j0 + j) * ldc;
-      dst[r0] = (beta == 0.0) ? (double)acc0[j] : fma(beta, dst[r0], (double)acc0[j]);
-      if (v1) dst[r1] = (beta == 0.0) ? (double)acc1[j] : fma(beta, dst[r1], (double)acc1[j]);
+      const double x0 = as_f64<INT>(acc0[j]), x1 = as_f64<INT>(acc1[j]);
+      if constexpr (kOld) {
+        dst[r0] = (beta == 0.0) ? x0 : fma(beta, old0[j], x0);
+        if (v1) dst[r1] = (beta == 0.0) ? x1 : fma(beta, old1[j], x1);
+      } else {
+        dst[r0] = (beta == 0.0) ? x0 : fma(beta, dst[r0], x0);
+        if (v1) dst[r1] = (beta == 0.0) ? x1 : fma(beta, dst[r1], x1);
+      }
     }
   }
 }
@@ -611,7 +661,7 @@ void launch_gram(const double *A, long long lda, long long bsa, int p, const dou
   const int BP = BQ == 1 ? pow2(p, 1, 16) : (BQ == 2 ? pow2(p, 2, 8) : 4);
   const int npb = ((p + BP - 1) / BP) * ((q + BQ - 1) / BQ);
   const int V = BP * BQ;
-  int nchunk = gram_chunks(nrows, batch, npb);
+  int nchunk = gram_chunks(nrows, batch, npb, low);
   // partial sums fit the scratch; sized with 16 values per block at least, so that
   // batch * npb also stays below the ticket count (one per 16 doubles of capacity)
   const long long cap = scr.capacity / ((long long)batch * npb * (V > 16 ? V : 16));
@@ -638,16 +688,20 @@ void launch_gram(const double *A, long long lda, long long bsa, int p, const dou
 #undef TPS_GRAM
 }
 
-// Resident CTAs per SM of k_update<T, BQ> (queried once per instantiation).
-int update_occupancy(bool low, int BQ) {
-  static int occ[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+// Resident CTAs per SM of the k_update variants (queried once): FP64, FP32 products with the
+// hardware conversions, and with integer ones.
+int update_occupancy(int kind, int BQ) {
+  static int occ[3][4] = {};
   static std::once_flag once;
   std::call_once(once, [] {
-    const void *fn[2][4] = {{(const void *)k_update<double, 1>, (const void *)k_update<double, 2>,
-                             (const void *)k_update<double, 4>, (const void *)k_update<double, 8>},
-                            {(const void *)k_update<float, 1>, (const void *)k_update<float, 2>,
-                             (const void *)k_update<float, 4>, (const void *)k_update<float, 8>}};
-    for (int t = 0; t < 2; ++t)
+    const void *fn[3][4] = {
+        {(const void *)k_update<double, 1, false>, (const void *)k_update<double, 2, false>,
+         (const void *)k_update<double, 4, false>, (const void *)k_update<double, 8, false>},
+        {(const void *)k_update<float, 1, false>, (const void *)k_update<float, 2, false>,
+         (const void *)k_update<float, 4, false>, (const void *)k_update<float, 8, false>},
+        {(const void *)k_update<float, 1, true>, (const void *)k_update<float, 2, true>,
+         (const void *)k_update<float, 4, true>, (const void *)k_update<float, 8, true>}};
+    for (int t = 0; t < 3; ++t)
       for (int b = 0; b < 4; ++b) {
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn[t][b], GT, 0) != cudaSuccess)
@@ -655,7 +709,7 @@ int update_occupancy(bool low, int BQ) {
         occ[t][b] = n < 1 ? 1 : n;
       }
   });
-  return occ[low ? 1 : 0][BQ == 1 ? 0 : (BQ == 2 ? 1 : (BQ == 4 ? 2 : 3))];
+  return occ[kind][BQ == 1 ? 0 : (BQ == 2 ? 1 : (BQ == 4 ? 2 : 3))];
 }
 
 void launch_update(const double *A, long long lda, long long bsa, int p, const double *Y, int ldy,
@@ -676,7 +730,12 @@ void launch_update(const double *A, long long lda, long long bsa, int p, const d
   const int zb = (q + BQ - 1) / BQ;
   // one wave: as many CTAs as fit on the SMs at once (over all systems and column blocks),
   // each striding over the rows
-  const int occ = update_occupancy(low, BQ);
+  // Integer conversions where the rows are many and the FP64 pipe would bound the stream
+  // (3 systems of 5.3 M rows: q = 4 in 83 us instead of 115, q = 2 in 72 instead of 86); a
+  // short input waits for latencies, which they lengthen (131,584 rows, q = 8: 18.1 instead of
+  // 15.6), and q = 1 gains nothing (173 us either way, 0.8 of HBM).
+  const bool ints = low && q > 1 && nrows >= (1 << 20);
+  const int occ = update_occupancy(low ? (ints ? 2 : 1) : 0, BQ);
   long long gx = (nrows + 2 * GT - 1) / (2 * GT);
   const long long wave = std::max(1LL, 152LL * occ / ((long long)batch * zb));
   if (gx > 8 * wave) gx = wave;  // short inputs keep a CTA per 512 rows
@@ -687,14 +746,19 @@ void launch_update(const double *A, long long lda, long long bsa, int p, const d
     const double bt = i0 == 0 ? beta : 1.0;
     const double *Ai = A + (long long)i0 * lda;
     count_launch();
-#define TPS_UPD(T, bq)                                                                       \
-  launch_pdl(k_update<T, bq>, grid, GT, 0, s, Ai, lda, bsa, pp, Y + i0, ldy, bsy, q, alpha, bt, C, \
-             ldc,                                                                                  \
-                                      bsc, nrows, need)
-    if (low)
-      BQ == 8 ? TPS_UPD(float, 8) : (BQ == 4 ? TPS_UPD(float, 4) : (BQ == 2 ? TPS_UPD(float, 2) : TPS_UPD(float, 1)));
+#define TPS_UPD(T, bq, in)                                                                    \
+  launch_pdl(k_update<T, bq, in>, grid, GT, 0, s, Ai, lda, bsa, pp, Y + i0, ldy, bsy, q, alpha, \
+             bt, C, ldc, bsc, nrows, need)
+#define TPS_UPDQ(T, in)                                            \
+  (BQ == 8 ? TPS_UPD(T, 8, in)                                     \
+           : (BQ == 4 ? TPS_UPD(T, 4, in) : (BQ == 2 ? TPS_UPD(T, 2, in) : TPS_UPD(T, 1, in))))
+    if (ints)
+      TPS_UPDQ(float, true);
+    else if (low)
+      TPS_UPDQ(float, false);
     else
-      BQ == 8 ? TPS_UPD(double, 8) : (BQ == 4 ? TPS_UPD(double, 4) : (BQ == 2 ? TPS_UPD(double, 2) : TPS_UPD(double, 1)));
+      TPS_UPDQ(double, false);
+#undef TPS_UPDQ
 #undef TPS_UPD
   }
 }
@@ -707,21 +771,19 @@ k_col_norms2(const double *__restrict__ A, long long lda, long long nrows, int n
              double *__restrict__ partial, unsigned *__restrict__ count, double *__restrict__ out) {
   pdl_entry();
   const int chunk = blockIdx.x, c = blockIdx.y;
-  const long long rows_per = (nrows + nchunk - 1) / nchunk;
-  const long long r0 = (long long)chunk * rows_per;
-  const long long r1 = r0 + rows_per < nrows ? r0 + rows_per : nrows;
+  const long long step = (long long)nchunk * GT;  // interleaved, as in k_gram
   const double *a = A + (long long)c * lda;
   // four independent loads in flight per thread
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  long long r = r0 + threadIdx.x;
-  for (; r + 3 * GT < r1; r += 4 * GT) {
-    const double x0 = a[r], x1 = a[r + GT], x2 = a[r + 2 * GT], x3 = a[r + 3 * GT];
+  long long r = (long long)chunk * GT + threadIdx.x;
+  for (; r + 3 * step < nrows; r += 4 * step) {
+    const double x0 = a[r], x1 = a[r + step], x2 = a[r + 2 * step], x3 = a[r + 3 * step];
     s0 = fma(x0, x0, s0);
     s1 = fma(x1, x1, s1);
     s2 = fma(x2, x2, s2);
     s3 = fma(x3, x3, s3);
   }
-  for (; r < r1; r += GT) s0 = fma(a[r], a[r], s0);
+  for (; r < nrows; r += step) s0 = fma(a[r], a[r], s0);
   double v = (s0 + s1) + (s2 + s3);
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   __shared__ double red[GT / 32];

@@ -33,6 +33,20 @@ __device__ __forceinline__ float f32_of_f64(double x) {
   return __uint_as_float(r);
 }
 
+// x rounded to the nearest FP32 (ties away from zero): the rounding unit is added to the bits,
+// which are then moved and the exponent rebased, nine integer instructions.  Outside the FP32
+// normal range, zeros included, the hardware conversion does it, under a branch that the
+// compiler must not turn into a conversion of every element.
+__device__ __forceinline__ float f32_near(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) + (1ull << 28);
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  // FP64 exponent 897 .. 1150 (FP32 1 .. 254); 896 mod 512 in the nine exponent bits kept
+  float f = __uint_as_float((__funnelshift_l(lo, hi, 3) - (384u << 23)) | (hi & 0x80000000u));
+  if ((hi & 0x7FFFFFFFu) - (897u << 20) >= (254u << 20))
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(x));
+  return f;
+}
+
 // f exactly as FP64 (FP32 subnormals, below 1.2e-38, flush to a signed zero).
 __device__ __forceinline__ double f64_of_f32(float f) {
   const unsigned u = __float_as_uint(f);

@@ -66,6 +66,31 @@ inline GemmArgs base_args() {
 
 constexpr int TK = 16;
 
+// The epilogue of element (m, n) of batch z, c its product, th its theta.
+template <typename Acc, typename TC>
+__device__ __forceinline__ void finish_element(const GemmArgs &g, long long z, int m, int n, Acc c,
+                                               double th) {
+  TC *dst = static_cast<TC *>(g.C) + z * g.bsc + (long long)m * g.ldc + n;
+  if (g.epi == EPI_HAPPLY) {
+    const Acc v = static_cast<const Acc *>(g.V)[(z % g.vmod) * g.vbs + (long long)m * g.ldv + n];
+    const Acc p = static_cast<const Acc *>(g.E.p)[z * g.E.bs + (long long)m * g.E.rs + n];
+    c = fma(v - static_cast<Acc>(th), p, c);
+  } else if (g.epi == EPI_DIVIDE2 || g.epi == EPI_DIVIDE4) {
+    const Acc *lamM = static_cast<const Acc *>(g.lamM), *lamN = static_cast<const Acc *>(g.lamN);
+    if (g.epi == EPI_DIVIDE2) {
+      c = c / (lamM[m] + lamN[n] - static_cast<Acc>(g.sigma));
+    } else {
+      const Acc *lam2 = static_cast<const Acc *>(g.lam2), *lam3 = static_cast<const Acc *>(g.lam3);
+      const int n23 = g.n2 * g.n3;
+      const Acc d = lamM[m] + lamN[n / n23] + lam2[(n / g.n3) % g.n2] + lam3[n % g.n3];
+      c = c / (d - static_cast<Acc>(g.sigma));
+    }
+  } else if (g.epi == EPI_ACCUM) {
+    c += static_cast<Acc>(*dst);
+  }
+  *dst = static_cast<TC>(c);
+}
+
 template <typename Acc, typename TA, typename TB, typename TC, int TM, int TN, int R = 4>
 __global__ void __launch_bounds__((TM / R) * (TN / R))
 k_gemm(const GemmArgs g) {
@@ -165,9 +190,6 @@ k_gemm(const GemmArgs g) {
 
   double th = 0.0;
   if (g.epi == EPI_HAPPLY) th = g.theta ? g.theta[z / g.theta_div] : g.theta0;
-  const Acc *lamM = static_cast<const Acc *>(g.lamM), *lamN = static_cast<const Acc *>(g.lamN);
-  const Acc *lam2 = static_cast<const Acc *>(g.lam2), *lam3 = static_cast<const Acc *>(g.lam3);
-  TC *Cz = static_cast<TC *>(g.C) + z * g.bsc;
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const int m = m0 + tm * R + i;
@@ -175,25 +197,87 @@ k_gemm(const GemmArgs g) {
 #pragma unroll
     for (int j = 0; j < R; ++j) {
       const int n = n0 + tn * R + j;
-      if (n >= g.Nc) continue;
-      Acc c = acc[i][j];
-      TC *dst = Cz + (long long)m * g.ldc + n;
-      if (g.epi == EPI_HAPPLY) {
-        const Acc v = static_cast<const Acc *>(g.V)[(z % g.vmod) * g.vbs + (long long)m * g.ldv + n];
-        const Acc p = static_cast<const Acc *>(g.E.p)[z * g.E.bs + (long long)m * g.E.rs + n];
-        c = fma(v - static_cast<Acc>(th), p, c);
-      } else if (g.epi == EPI_DIVIDE2) {
-        c = c / (lamM[m] + lamN[n] - static_cast<Acc>(g.sigma));
-      } else if (g.epi == EPI_DIVIDE4) {
-        const int n23 = g.n2 * g.n3;
-        const Acc d = lamM[m] + lamN[n / n23] + lam2[(n / g.n3) % g.n2] + lam3[n % g.n3];
-        c = c / (d - static_cast<Acc>(g.sigma));
-      } else if (g.epi == EPI_ACCUM) {
-        c += static_cast<Acc>(*dst);
-      }
-      *dst = static_cast<TC>(c);
+      if (n < g.Nc) finish_element<Acc, TC>(g, z, m, n, acc[i][j], th);
     }
   }
+}
+
+// FP64 products without shared-memory tiles.  GB300's FP64 pipe takes a warp instruction per
+// ~64 cycles of a scheduler, so a warp's FMA leaves time for its loads to come from L1 and L2,
+// whatever their reuse; what matters is that every scheduler of every SM has warps with FMAs to
+// issue.  A CTA computes (32 / LC) R x LC outputs, R per lane of each of its 8 warps, which
+// split K between them (adjacent pieces, added in order at the end: 7 FP64 additions per
+// output).  H-apply, tiled -> direct: 64 x 64, 1 vector 79 -> 9 us (one 64-thread CTA of the
+// tiled kernel runs all of K on two schedulers); 128 x 128, 4 vectors 150 -> 37; 512 x 512, 8
+// vectors 3610 -> 3480, 0.97 of the pipe.
+constexpr int kDirectWarps = 8;
+template <int R, int LC>
+__global__ void __launch_bounds__(32 * kDirectWarps)
+k_gemm_direct(const GemmArgs g) {
+  constexpr int LR = 32 / LC;
+  __shared__ double red[kDirectWarps][R][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tiles = g.tiles_m * g.tiles_n;
+  const long long z = blockIdx.x / tiles;
+  const int t = (int)(blockIdx.x % tiles);
+  const int m0 = (t / g.tiles_n) * (LR * R) + lane / LC, n = (t % g.tiles_n) * LC + lane % LC;
+  const int nc = n < g.Nc ? n : g.Nc - 1;  // lanes and rows beyond the edge repeat the last one
+  double acc[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) acc[i] = 0.0;
+  for (int ph = 0; ph < g.nphase; ++ph) {
+    const int K = g.K[ph];
+    const int k0 = (int)((long long)K * warp / kDirectWarps);
+    const int k1 = (int)((long long)K * (warp + 1) / kDirectWarps);
+    const double *Bp = static_cast<const double *>(g.B[ph].p) + z * g.B[ph].bs + nc;
+    const double *Ap[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int m = m0 + LR * i < g.M ? m0 + LR * i : g.M - 1;
+      Ap[i] = static_cast<const double *>(g.A[ph].p) + z * g.A[ph].bs + (long long)m * g.A[ph].rs;
+    }
+    const long long brs = g.B[ph].rs;
+    int k = k0;
+    for (; k + 4 <= k1; k += 4) {
+      double b[4], a[R][4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        b[u] = Bp[(k + u) * brs];
+#pragma unroll
+        for (int i = 0; i < R; ++i) a[i][u] = Ap[i][k + u];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i] = fma(a[i][u], b[u], acc[i]);
+    }
+    for (; k < k1; ++k) {
+      const double b = Bp[k * brs];
+#pragma unroll
+      for (int i = 0; i < R; ++i) acc[i] = fma(Ap[i][k], b, acc[i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) red[warp][i][lane] = acc[i];
+  __syncthreads();
+  if (warp >= R) return;
+  double c = red[0][warp][lane];
+#pragma unroll
+  for (int w = 1; w < kDirectWarps; ++w) c += red[w][warp][lane];
+  const int m = m0 + LR * warp;
+  if (m >= g.M || n >= g.Nc) return;
+  const double th = g.epi != EPI_HAPPLY ? 0.0 : g.theta ? g.theta[z / g.theta_div] : g.theta0;
+  finish_element<double, double>(g, z, m, n, c, th);
+}
+
+template <int R, int LC>
+void run_direct(GemmArgs g, cudaStream_t s) {
+  g.tiles_m = (g.M + 32 / LC * R - 1) / (32 / LC * R);
+  g.tiles_n = (g.Nc + LC - 1) / LC;
+  const long long blocks = (long long)g.batch * g.tiles_m * g.tiles_n;
+  if (blocks <= 0) return;
+  count_launch();
+  k_gemm_direct<R, LC><<<(unsigned)blocks, 32 * kDirectWarps, 0, s>>>(g);
 }
 
 // Tile choice: minimise padded work plus a one-tile-per-SM imbalance allowance,
@@ -272,6 +356,21 @@ TileCache &tile_cache();
 
 template <typename Acc, typename TA, typename TB, typename TC>
 void gemm(GemmArgs g, cudaStream_t s) {
+  if constexpr (sizeof(Acc) == 8) {
+    // Many outputs of a short K keep the tiled kernel: splitting K costs 7 additions per output
+    // (2D H-apply of 2 vectors at 48^4, 10.6 M outputs a launch: tiled 3.62 ms, direct 4.55; at
+    // 48^2 x 24^2, 2.7 M outputs, 1.04 and 0.93).  Otherwise direct, with fewer outputs per
+    // lane while that leaves CTAs for two per SM; 32 columns per warp where rows are that long
+    // (24^4, 4 vectors: 328 us, 369 with 8).
+    const long long out = (long long)g.M * g.Nc * g.batch;
+    const int K = g.K[0] + (g.nphase > 1 ? g.K[1] : 0);
+    if (out < (1LL << 22) || K > 128) {
+      if (out <= 32 * 304) return run_direct<1, 8>(g, s);
+      if (out <= 64 * 304) return run_direct<2, 8>(g, s);
+      if (g.Nc < 256) return run_direct<4, 8>(g, s);
+      return run_direct<4, 32>(g, s);
+    }
+  }
   int tm, tn;
   pick_tiles(g, tm, tn);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
