@@ -374,3 +374,15 @@ def test_apply_prec_tf32_rejects_2d_modes(n):
     with pytest.raises(tps.TpsError):
         ctx.apply_prec(x, y, -0.5, dtype=tps.TF32_TC)
     ctx.close()
+
+
+@pytest.mark.parametrize("n,nvec", [((96, 100), 1), ((98, 100), 1), ((140, 138), 1),
+                                    ((142, 138), 1), ((6, 512), 6), ((6, 514), 7), ((50, 260), 2),
+                                    ((4, 258), 20)])
+def test_apply_h_1d_around_the_direct_kernels_limits(n, nvec):
+    # output counts on both sides of the limits between one, two and four outputs per lane, and
+    # rows of 256 points and more (32 columns per warp) that fill no tile
+    require_gpu()
+    P = problem_1d(20.0, 1.0, 1.0, n, (20.0, 15.0), 1.0, 1.0)
+    ctx = make_ctx_1d(20.0, 1.0, n, (20.0, 15.0), 1.0, 1.0)
+    _check_h(P, ctx, nvec, 0.3, seed=5)
