@@ -42,137 +42,185 @@ __device__ __forceinline__ float gelu_grad(float z) {
          z * 0.39894228040143268f * expf(-0.5f * z * z);
 }
 
-// Y[B][out] = X[B][in] W[in][out] + b, Z = pre-activation kept for the backward pass,
-// A = GELU(Z) (act = 1) or Z (act = 0).  W is FP32 or BF16.  32 x 32 output tile per
-// CTA, 256 threads, 4 outputs each.
-template <typename TW>
-__global__ void __launch_bounds__(256)
-k_linear_fwd(const float *__restrict__ X, int B, int in, const TW *__restrict__ W,
-             const float *__restrict__ bias, int out, int act, float *__restrict__ Z,
-             float *__restrict__ A) {
-  __shared__ float xs[kTile][kTile + 1];
-  __shared__ float ws[kTile][kTile + 1];
-  const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;  // ty in 0..7
-  const int r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int k0 = 0; k0 < in; k0 += kTile) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int rr = ty + 8 * j;
-      const int r = r0 + rr, k = k0 + tx;
-      xs[rr][tx] = (r < B && k < in) ? X[(long long)r * in + k] : 0.f;
-      const int kk = k0 + rr, c = c0 + tx;
-      ws[rr][tx] = (kk < in && c < out) ? (float)W[(long long)kk * out + c] : 0.f;
+// The products of the forward and backward passes, C[m][n] = sum_k A(m, k) B(k, n).  They are
+// small (a batch of some hundred rows, 256-wide layers): few tiles and long chains of loads,
+// barriers and short inner loops.  A CTA of 512 threads computes a 32 x 32 tile; eight groups of
+// 64 threads take every eighth slab of 16 k, each with its own shared-memory slab and barrier
+// and the next slab's loads in flight, 4 x 4 outputs per thread, and add their sums at the end.
+// (256 threads on one slab of 32 k at a time, 4 outputs each: 71 us for the 256 x 256 x 1024
+// product of the last layer's input gradient.)
+constexpr int kGroups = 8, kSlab = 16, kLd = kTile + 4;
+
+template <bool AK, bool BK, typename TB>  // AK: A's k is contiguous (else m); BK: B's k (else n)
+struct TileGemm {
+  const float *A;
+  const TB *B;
+  int M, N, K, lda, ldb;
+
+  __device__ __forceinline__ static void place(bool kc, int t, int e, int &row, int &k) {
+    if (kc) {  // 32 rows x 2 halves of the slab
+      row = t >> 1;
+      k = (t & 1) * 8 + e;
+    } else {  // 16 k x 4 quarters of the rows
+      row = (t & 3) * 8 + e;
+      k = t >> 2;
     }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kTile; ++k) {
-      const float w = ws[k][tx];
+  }
+  __device__ __forceinline__ void load(int t, int m0, int n0, int k0, float (&a)[8],
+                                       float (&b)[8]) const {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[j] = fmaf(xs[ty + 8 * j][k], w, acc[j]);
+    for (int e = 0; e < 8; ++e) {
+      int r, k;
+      place(AK, t, e, r, k);
+      a[e] = (m0 + r < M && k0 + k < K)
+                 ? A[AK ? (long long)(m0 + r) * lda + k0 + k : (long long)(k0 + k) * lda + m0 + r]
+                 : 0.f;
+      place(BK, t, e, r, k);
+      b[e] = (n0 + r < N && k0 + k < K)
+                 ? (float)B[BK ? (long long)(n0 + r) * ldb + k0 + k
+                               : (long long)(k0 + k) * ldb + n0 + r]
+                 : 0.f;
+    }
+  }
+  // The tile's sums in sh[m][n] (32 x 32) for all threads; bsum (nullable): sum_k B(k, n) of the
+  // tile's columns.  sh: kTileSmem bytes, the slabs first and then the groups' sums.
+  __device__ __forceinline__ void run(int m0, int n0, float *sh, float *bsum) const {
+    const int g = threadIdx.x >> 6, t = threadIdx.x & 63, tm = t >> 3, tn = t & 7;
+    float(*as)[kLd] = reinterpret_cast<float(*)[kLd]>(sh + g * 2 * kSlab * kLd);
+    float(*bs)[kLd] = as + kSlab;
+    float acc[4][4] = {}, bacc[4] = {};
+    float a[8], b[8];
+    load(t, m0, n0, g * kSlab, a, b);
+    for (int k0 = g * kSlab; k0 < K; k0 += kGroups * kSlab) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        int r, k;
+        place(AK, t, e, r, k);
+        as[k][r] = a[e];
+        place(BK, t, e, r, k);
+        bs[k][r] = b[e];
+      }
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + g) : "memory");
+      load(t, m0, n0, k0 + kGroups * kSlab, a, b);  // zeros past the end
+#pragma unroll
+      for (int k = 0; k < kSlab; ++k) {
+        const float4 x = *reinterpret_cast<const float4 *>(&as[k][tm * 4]);
+        const float4 y = *reinterpret_cast<const float4 *>(&bs[k][tn * 4]);
+        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xs[i], ys[j], acc[i][j]);
+        if (bsum && tm == 0)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) bacc[j] += ys[j];
+      }
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + g) : "memory");
+    }
+    __shared__ float bred[kGroups][kTile];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        sh[(g * kTile + tm * 4 + i) * kTile + tn * 4 + j] = acc[i][j];
+    if (bsum && tm == 0)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) bred[g][tn * 4 + j] = bacc[j];
+    __syncthreads();
+    for (int e = threadIdx.x; e < kTile * kTile; e += 64 * kGroups) {
+      float v = sh[e];
+#pragma unroll
+      for (int h = 1; h < kGroups; ++h) v += sh[h * kTile * kTile + e];
+      sh[e] = v;
+    }
+    if (bsum && threadIdx.x < kTile) {
+      float v = 0.f;
+#pragma unroll
+      for (int h = 0; h < kGroups; ++h) v += bred[h][threadIdx.x];
+      bsum[threadIdx.x] = v;
     }
     __syncthreads();
   }
-  const int c = c0 + tx;
-  if (c >= out) return;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int r = r0 + ty + 8 * j;
-    if (r >= B) continue;
-    const float z = acc[j] + bias[c];
+};
+constexpr size_t kTileSmem = sizeof(float) * kGroups * 2 * kSlab * kLd;
+static_assert(2 * kSlab * kLd >= kTile * kTile, "the sums fit where the slabs were");
+
+// Y[B][out] = X[B][in] W[in][out] + b, Z = pre-activation kept for the backward pass,
+// A = GELU(Z) (act = 1) or Z (act = 0).  W is FP32 or BF16.
+template <typename TW>
+__global__ void __launch_bounds__(64 * kGroups)
+k_linear_fwd(const float *__restrict__ X, int B, int in, const TW *__restrict__ W,
+             const float *__restrict__ bias, int out, int act, float *__restrict__ Z,
+             float *__restrict__ A) {
+  extern __shared__ float sh[];
+  const int r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
+  const TileGemm<true, false, TW> g = {X, W, B, out, in, in, out};
+  g.run(r0, c0, sh, nullptr);
+  for (int e = threadIdx.x; e < kTile * kTile; e += 64 * kGroups) {
+    const int r = r0 + e / kTile, c = c0 + e % kTile;
+    if (r >= B || c >= out) continue;
+    const float z = sh[e] + bias[c];
     if (Z) Z[(long long)r * out + c] = z;
     A[(long long)r * out + c] = act ? gelu(z) : z;
   }
 }
 
-// dW[in][out] = X^T dZ, db[out] = sum_rows dZ (one CTA column block, all rows).
-__global__ void __launch_bounds__(256)
+// dW[in][out] = X^T dZ, db[out] = sum_rows dZ.
+__global__ void __launch_bounds__(64 * kGroups)
 k_linear_wgrad(const float *__restrict__ X, int B, int in, const float *__restrict__ dZ, int out,
                float *__restrict__ dW, float *__restrict__ db) {
-  __shared__ float xs[kTile][kTile + 1];
-  __shared__ float gs[kTile][kTile + 1];
-  const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
+  extern __shared__ float sh[];
+  __shared__ float bsum[kTile];
   const int i0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  float bacc = 0.f;
-  for (int r0 = 0; r0 < B; r0 += kTile) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int rr = ty + 8 * j;
-      const int r = r0 + rr;
-      xs[rr][tx] = (r < B && i0 + tx < in) ? X[(long long)r * in + i0 + tx] : 0.f;
-      gs[rr][tx] = (r < B && c0 + tx < out) ? dZ[(long long)r * out + c0 + tx] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int r = 0; r < kTile; ++r) {
-      const float g = gs[r][tx];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[j] = fmaf(xs[r][ty + 8 * j], g, acc[j]);
-      if (ty == 0 && blockIdx.y == 0) bacc += g;
-    }
-    __syncthreads();
+  const TileGemm<false, false, float> g = {X, dZ, in, out, B, in, out};
+  g.run(i0, c0, sh, blockIdx.y == 0 ? bsum : nullptr);
+  for (int e = threadIdx.x; e < kTile * kTile; e += 64 * kGroups) {
+    const int i = i0 + e / kTile, c = c0 + e % kTile;
+    if (i < in && c < out) dW[(long long)i * out + c] = sh[e];
   }
-  const int c = c0 + tx;
-  if (c >= out) return;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int i = i0 + ty + 8 * j;
-    if (i < in) dW[(long long)i * out + c] = acc[j];
-  }
-  if (ty == 0 && blockIdx.y == 0) db[c] = bacc;
+  if (blockIdx.y == 0 && threadIdx.x < kTile && c0 + threadIdx.x < out)
+    db[c0 + threadIdx.x] = bsum[threadIdx.x];
 }
 
 // dX[B][in] = (dZ W^T) [B][in], then (prev_act) dZ_prev = dX * GELU'(Z_prev) in place.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(64 * kGroups)
 k_linear_xgrad(const float *__restrict__ dZ, int B, int out, const float *__restrict__ W, int in,
                const float *__restrict__ Zprev, float *__restrict__ dX) {
-  __shared__ float gs[kTile][kTile + 1];
-  __shared__ float ws[kTile][kTile + 1];
-  const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
+  extern __shared__ float sh[];
   const int r0 = blockIdx.y * kTile, i0 = blockIdx.x * kTile;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int c0 = 0; c0 < out; c0 += kTile) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int rr = ty + 8 * j;
-      gs[rr][tx] = (r0 + rr < B && c0 + tx < out) ? dZ[(long long)(r0 + rr) * out + c0 + tx] : 0.f;
-      // ws[c][i] = W[i][c]
-      ws[tx][rr] = (i0 + rr < in && c0 + tx < out) ? W[(long long)(i0 + rr) * out + c0 + tx] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int c = 0; c < kTile; ++c) {
-      const float w = ws[c][tx];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[j] = fmaf(gs[ty + 8 * j][c], w, acc[j]);
-    }
-    __syncthreads();
-  }
-  const int i = i0 + tx;
-  if (i >= in) return;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int r = r0 + ty + 8 * j;
-    if (r >= B) continue;
-    const long long e = (long long)r * in + i;
-    dX[e] = acc[j] * (Zprev ? gelu_grad(Zprev[e]) : 1.f);
+  const TileGemm<true, true, float> g = {dZ, W, B, in, out, out, out};
+  g.run(r0, i0, sh, nullptr);
+  for (int e = threadIdx.x; e < kTile * kTile; e += 64 * kGroups) {
+    const int r = r0 + e / kTile, i = i0 + e % kTile;
+    if (r >= B || i >= in) continue;
+    const long long at = (long long)r * in + i;
+    dX[at] = sh[e] * (Zprev ? gelu_grad(Zprev[at]) : 1.f);
   }
 }
 
 // Per sample: P = C^T D (px x py), loss = 1 - <P,T>^2/(|P|^2 |T|^2), and dL/d(output)
-// into G (same layout as the output row: C then D).  One CTA per sample; loss[s] FP64.
+// into G (same layout as the output row: C then D).  One CTA per sample; loss[s] FP64.  stage:
+// C and D are kept in shared memory and the rows of P padded by one, so that the threads of the
+// gradient sums, each on a row of dL/dP, meet in no bank (37 us without for 256 samples of
+// 16 x (32 + 32)).
 __global__ void __launch_bounds__(256)
 k_cosine_loss(const float *__restrict__ out, int R, int px, int py, const float *__restrict__ T,
-              float *__restrict__ G, double *__restrict__ loss, float inv_batch) {
+              float *__restrict__ G, double *__restrict__ loss, float inv_batch, int stage) {
   extern __shared__ float sh[];
-  float *P = sh;                 // px * py
-  float *dP = P + px * py;       // px * py
+  const int ld = py + stage;
+  float *P = sh;  // px * ld, then dL/dP in its place
   __shared__ float red[3][8];
   __shared__ float coef[2];
   const int s = blockIdx.x, tid = threadIdx.x;
   const int dout = R * (px + py);
   const float *C = out + (long long)s * dout;
+  if (stage) {
+    float *cd = P + px * ld;
+    for (int e = tid; e < dout; e += blockDim.x) cd[e] = C[e];
+    C = cd;
+    __syncthreads();
+  }
   const float *D = C + R * px;
   const float *Ts = T + (long long)s * px * py;
   float pt = 0.f, pp = 0.f, tt = 0.f;
@@ -180,7 +228,7 @@ k_cosine_loss(const float *__restrict__ out, int R, int px, int py, const float 
     const int a = e / py, b = e % py;
     float v = 0.f;
     for (int r = 0; r < R; ++r) v = fmaf(C[r * px + a], D[r * py + b], v);
-    P[e] = v;
+    P[a * ld + b] = v;
     const float t = Ts[e];
     pt = fmaf(v, t, pt);
     pp = fmaf(v, v, pp);
@@ -211,20 +259,23 @@ k_cosine_loss(const float *__restrict__ out, int R, int px, int py, const float 
     coef[1] = 2.f * a * a / (den * fmaxf(b, 1e-30f)) * inv_batch;
   }
   __syncthreads();
-  for (int e = tid; e < px * py; e += blockDim.x) dP[e] = coef[0] * Ts[e] + coef[1] * P[e];
+  for (int e = tid; e < px * py; e += blockDim.x) {
+    float *p = P + e / py * ld + e % py;
+    *p = coef[0] * Ts[e] + coef[1] * *p;
+  }
   __syncthreads();
   float *Gs = G + (long long)s * dout;
   // dC[r][a] = sum_b dP[a][b] D[r][b],  dD[r][b] = sum_a dP[a][b] C[r][a]
   for (int e = tid; e < R * px; e += blockDim.x) {
     const int r = e / px, a = e % px;
     float v = 0.f;
-    for (int b = 0; b < py; ++b) v = fmaf(dP[a * py + b], D[r * py + b], v);
+    for (int b = 0; b < py; ++b) v = fmaf(P[a * ld + b], D[r * py + b], v);
     Gs[e] = v;
   }
   for (int e = tid; e < R * py; e += blockDim.x) {
     const int r = e / py, b = e % py;
     float v = 0.f;
-    for (int a = 0; a < px; ++a) v = fmaf(dP[a * py + b], C[r * px + a], v);
+    for (int a = 0; a < px; ++a) v = fmaf(P[a * ld + b], C[r * px + a], v);
     Gs[R * px + e] = v;
   }
 }
@@ -401,6 +452,8 @@ struct tps_ws {
 namespace {
 
 using tps::mlp::kLayers;
+constexpr int kT = 64 * tps::mlp::kGroups;       // threads and dynamic shared memory of the
+constexpr size_t kSh = tps::mlp::kTileSmem;      // layers' products
 
 int ws_error(tps_ws *ws, int code, const std::string &msg) {
   if (ws) ws->err = msg;
@@ -468,11 +521,11 @@ void forward(tps_ws *ws, int B, bool bf16, cudaStream_t s) {
     const int act = l < kLayers - 1 ? 1 : 0;
     tps::count_launch();
     if (bf16)
-      tps::mlp::k_linear_fwd<__nv_bfloat16><<<grid, 256, 0, s>>>(
+      tps::mlp::k_linear_fwd<__nv_bfloat16><<<grid, kT, kSh, s>>>(
           ws->A[l], B, in, ws->wb + ws->woff[l], ws->w + ws->boff[l], out, act, ws->Z[l],
           ws->A[l + 1]);
     else
-      tps::mlp::k_linear_fwd<float><<<grid, 256, 0, s>>>(ws->A[l], B, in, ws->w + ws->woff[l],
+      tps::mlp::k_linear_fwd<float><<<grid, kT, kSh, s>>>(ws->A[l], B, in, ws->w + ws->woff[l],
                                                          ws->w + ws->boff[l], out, act, ws->Z[l],
                                                          ws->A[l + 1]);
   }
@@ -699,19 +752,21 @@ int tps_ws_loss_grad(tps_ws *ws, const float *X_dev, const float *T_dev, int B, 
                                   cudaMemcpyDeviceToDevice, stream));
   forward(ws, B, false, stream);
   // loss and dL/d(output) into dZa
-  const size_t shm = sizeof(float) * 2 * ws->px * ws->py;
+  const size_t plain = sizeof(float) * 2 * ws->px * ws->py;  // as many modes as before fit
+  const size_t staged = sizeof(float) * ((size_t)ws->px * (ws->py + 1) + ws->dims[kLayers]);
+  const int stage = staged <= (48u << 10) && plain <= (48u << 10) ? 1 : 0;
   tps::count_launch();
-  tps::mlp::k_cosine_loss<<<B, 256, shm, stream>>>(ws->A[kLayers], ws->R, ws->px, ws->py, T_dev,
-                                                   ws->dZa, ws->loss, 1.0f / B);
+  tps::mlp::k_cosine_loss<<<B, 256, stage ? staged : plain, stream>>>(
+      ws->A[kLayers], ws->R, ws->px, ws->py, T_dev, ws->dZa, ws->loss, 1.0f / B, stage);
   float *dz = ws->dZa, *dprev = ws->dZb;
   for (int l = kLayers - 1; l >= 0; --l) {
     const int in = ws->dims[l], out = ws->dims[l + 1];
     tps::count_launch();
-    tps::mlp::k_linear_wgrad<<<dim3((out + 31) / 32, (in + 31) / 32), 256, 0, stream>>>(
+    tps::mlp::k_linear_wgrad<<<dim3((out + 31) / 32, (in + 31) / 32), kT, kSh, stream>>>(
         ws->A[l], B, in, dz, out, ws->g + ws->woff[l], ws->g + ws->boff[l]);
     if (l > 0) {
       tps::count_launch();
-      tps::mlp::k_linear_xgrad<<<dim3((in + 31) / 32, (B + 31) / 32), 256, 0, stream>>>(
+      tps::mlp::k_linear_xgrad<<<dim3((in + 31) / 32, (B + 31) / 32), kT, kSh, stream>>>(
           dz, B, out, ws->w + ws->woff[l], in, ws->Z[l - 1], dprev);
       std::swap(dz, dprev);
     }
