@@ -29,8 +29,8 @@
 //                   by one bulk copy per operand; levels lie side by side in tensor memory, so
 //                   a digit slice of F times all the digit slices of B it meets is one or two
 //                   MMAs (as in oz_mode.cu); writes the 64-bit sums;
-//   k_fold_combine  a thread per pair of representatives (r_x, r_y): unfolds both modes, adds the
-//                   potential term and writes the |G_x| |G_y| outputs.
+//   k_fold_combine  a thread per pair of representatives (r_x, r_y) and image of r_x: unfolds
+//                   both modes, adds the potential term and writes the |G_y| outputs.
 //
 // Measured, 8 vectors at 512 x 512: 119 us, 476 by the dense base-64 products.
 #include <cuda_fp16.h>
@@ -272,11 +272,18 @@ __global__ void __launch_bounds__(256) k_fold_split(const __grid_constant__ Spli
     if (lane < kLines) atomicMax(&ex[l], mx);
   }
   __syncthreads();
-  const int l = lane >> 1;
-  const unsigned raw = ex[l];
   if (tid < kLines && line0 + tid < g.nlines[d]) g.eL[d][line0 + tid] = (int)ex[tid] - 1022;
-  const double *x = tile + l * ld;
+  // the scaled integers in place of the values (each is used by every block of its images)
   const int bits = m.G == 4 ? 60 : m.G == 2 ? 61 : 62;
+  for (int k = warp; k < kLines; k += 8) {
+    const unsigned raw = ex[k];
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32)
+      tile[k * ld + i] = __longlong_as_double(scaled(tile[k * ld + i], raw, bits));
+  }
+  __syncthreads();
+  const int l = lane >> 1;
+  const long long *x = reinterpret_cast<const long long *>(tile) + l * ld;
   const int chunks = 2 * m.kc[0];  // the largest block's
   // the line's place in the operand layout
   const long long rt = (line0 + l) / kRows;
@@ -288,7 +295,7 @@ __global__ void __launch_bounds__(256) k_fold_split(const __grid_constant__ Spli
     for (int k = 0; k < 4; ++k)
 #pragma unroll
       for (int t = 0; t < 4; ++t)
-        a[k][t] = t < m.G && p0 + k < m.reps ? scaled(x[image_of(m, p0 + k, t)], raw, bits) : 0;
+        a[k][t] = t < m.G && p0 + k < m.reps ? x[image_of(m, p0 + k, t)] : 0;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       if (b >= m.G || c >= 2 * m.kc[b]) continue;
@@ -302,7 +309,7 @@ __global__ void __launch_bounds__(256) k_fold_split(const __grid_constant__ Spli
           for (int t = 0; t < 4; ++t) s += negative(b, t) ? -a[k][t] : a[k][t];
         } else if (r >= 0) {  // the representative n / 4 at position 0
           for (int t = 0; t < m.G; ++t) {
-            const long long y = scaled(x[image_of(m, r, t)], raw, bits);
+            const long long y = x[image_of(m, r, t)];
             s += negative(b, t) ? -y : y;
           }
         }
@@ -567,69 +574,56 @@ struct CombineArgs {
   double theta0;
 };
 
-// Lane = representative of y, so that every access is contiguous (or contiguous backwards).
+// A thread per pair of representatives and image of the one of x (threadIdx.y), adjacent lanes
+// on adjacent representatives of y, so that accesses are contiguous (or contiguous backwards).
+// The images of r_x read the same sums of the x mode, from L1.  (All images in one thread, 105
+// registers and a warp per row of representatives: 43 us at 512 x 512, 8 vectors.)
 template <int GX, int GY>
-__global__ void __launch_bounds__(128) k_fold_combine(const __grid_constant__ CombineArgs g) {
+__global__ void __launch_bounds__(64 * GX) k_fold_combine(const __grid_constant__ CombineArgs g) {
   if (threadIdx.x == 0 && threadIdx.y == 0) pdl_trigger();
   pdl_wait();
-  const int ry = blockIdx.x * 32 + threadIdx.x, rx = blockIdx.y * 4 + threadIdx.y;
-  const int v = blockIdx.z;
-  if (ry >= g.my.reps || rx >= g.mx.reps) return;
+  const int e = blockIdx.x * 64 + threadIdx.x, a = threadIdx.y, v = blockIdx.y;
+  const int rx = e / g.my.reps, ry = e - rx * g.my.reps;
+  if (rx >= g.mx.reps) return;
   const int nx = g.mx.n, ny = g.my.n;
+  const int ix = image_of(g.mx, rx, a);
+  for (int c = 0; c < a; ++c)
+    if (image_of(g.mx, rx, c) == ix) return;  // a point that the group leaves in place
   const double th = g.theta_dev ? g.theta_dev[v] : g.theta0;
-  const int eby = g.eBy[ry] - 62, ebx = g.eBx[rx] - 62;
-  int py[GY], px[GX], iy[GY], ix[GX];
+  const int ey = g.eLy[v * nx + ix] + g.eBy[ry] - 62, ebx = g.eBx[rx] - 62;
+  long long ty[GY], px[GX];
 #pragma unroll
   for (int b = 0; b < GY; ++b) {
-    py[b] = pos_of(g.my, b, ry);
-    iy[b] = image_of(g.my, ry, b);
+    const int p = pos_of(g.my, b, ry);
+    ty[b] = p >= 0 ? g.Ty[b][((long long)v * nx + ix) * g.ldy[b] + p] : 0;
   }
 #pragma unroll
-  for (int b = 0; b < GX; ++b) {
-    px[b] = pos_of(g.mx, b, rx);
-    ix[b] = image_of(g.mx, rx, b);
-  }
-  long long ty[GX][GY], tx[GX][GY];
+  for (int b = 0; b < GX; ++b) px[b] = pos_of(g.mx, b, rx);
+  int iy[GY];
 #pragma unroll
-  for (int a = 0; a < GX; ++a)
+  for (int t = 0; t < GY; ++t) {
+    iy[t] = image_of(g.my, ry, t);
+    bool dup = false;
 #pragma unroll
-    for (int b = 0; b < GY; ++b)
-      ty[a][b] = py[b] >= 0 ? g.Ty[b][((long long)v * nx + ix[a]) * g.ldy[b] + py[b]] : 0;
+    for (int c = 0; c < t; ++c) dup |= iy[c] == iy[t];
+    if (dup) continue;
+    const long long at = (long long)ix * ny + iy[t], col = (long long)v * ny + iy[t];
+    long long sy = 0, sx = 0;
 #pragma unroll
-  for (int b = 0; b < GX; ++b)
-#pragma unroll
-    for (int t = 0; t < GY; ++t)
-      tx[b][t] = px[b] >= 0 ? g.Tx[b][(long long)px[b] * g.ldx + (long long)v * ny + iy[t]] : 0;
-#pragma unroll
-  for (int a = 0; a < GX; ++a) {
-    const int ely = g.eLy[v * nx + ix[a]];
-    bool seen = false;  // a point that the group leaves in place is its own image
-#pragma unroll
-    for (int c = 0; c < a; ++c) seen |= ix[c] == ix[a];
-    if (seen) continue;
-#pragma unroll
-    for (int t = 0; t < GY; ++t) {
-      bool dup = false;
-#pragma unroll
-      for (int c = 0; c < t; ++c) dup |= iy[c] == iy[t];
-      if (dup) continue;
-      long long sy = 0, sx = 0;
-#pragma unroll
-      for (int b = 0; b < GY; ++b) sy += negative(b, t) ? -ty[a][b] : ty[a][b];
-#pragma unroll
-      for (int b = 0; b < GX; ++b) sx += negative(b, a) ? -tx[b][t] : tx[b][t];
-      const long long at = (long long)ix[a] * ny + iy[t];
-      const double y = round_int(sy, ely + eby);
-      const double x = round_int(sx, g.eLx[v * ny + iy[t]] + ebx);
-      g.out[(long long)v * g.N + at] =
-          fma(g.V[at] - th, g.psi[(long long)v * g.N + at], y) + x;
+    for (int b = 0; b < GX; ++b) {
+      const long long z = px[b] >= 0 ? g.Tx[b][px[b] * g.ldx + col] : 0;
+      sx += negative(b, a) ? -z : z;
     }
+#pragma unroll
+    for (int b = 0; b < GY; ++b) sy += negative(b, t) ? -ty[b] : ty[b];
+    const double y = round_int(sy, ey), x = round_int(sx, g.eLx[col] + ebx);
+    g.out[(long long)v * g.N + at] = fma(g.V[at] - th, g.psi[(long long)v * g.N + at], y) + x;
   }
 }
 
 template <int GX>
 cudaError_t launch_combine(const CombineArgs &c, dim3 grid, cudaStream_t s) {
-  const dim3 block(32, 4);
+  const dim3 block(64, GX);
   count_launch();
   switch (c.my.G) {
     case 1: return launch_pdl(k_fold_combine<GX, 1>, grid, block, 0, s, c);
@@ -813,7 +807,7 @@ cudaError_t apply(const Operator &o, const DevOperator &op, const double *psi, d
     c.theta0 = theta;
     c.out = O;
     c.N = op.N;
-    const dim3 grid((c.my.reps + 31) / 32, (c.mx.reps + 3) / 4, nv);
+    const dim3 grid((c.my.reps * c.mx.reps + 63) / 64, nv);
     e = c.mx.G == 4 ? launch_combine<4>(c, grid, s)
                     : c.mx.G == 2 ? launch_combine<2>(c, grid, s) : launch_combine<1>(c, grid, s);
     if (e != cudaSuccess) return e;
