@@ -92,6 +92,47 @@ __device__ __forceinline__ bool halving_writer(int lane) {  // one lane per valu
   return (lane & ((1 << (5 - used)) - 1)) == 0;
 }
 
+// The sum of acc over the threads of all nchunk CTAs that share `partial` and `count`, chunk c's
+// share first reduced in its CTA.  True in the last CTA to arrive, whose tot[0 .. V) then holds
+// the sums, added in an order that does not depend on scheduling; it re-arms the counter for
+// the next call on this stream.
+template <typename T, int V>
+__device__ __forceinline__ bool chunk_sums(T (&acc)[V], double *partial, unsigned *count, int c,
+                                           int nchunk, double (&tot)[GT]) {
+  warp_halving_sum<V>(acc);
+  __shared__ T red[GT / 32][V];
+  __shared__ unsigned ticket;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (halving_writer<V>(lane)) red[warp][halving_index<V>(lane)] = acc[0];
+  __syncthreads();
+  if (threadIdx.x < V) {
+    T v = T(0);
+    for (int w = 0; w < GT / 32; ++w) v += red[w][threadIdx.x];
+    partial[c * V + threadIdx.x] = (double)v;
+    __threadfence();  // this chunk's sums are visible before the ticket is taken
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) ticket = atomicAdd(count, 1u);
+  __syncthreads();
+  if (ticket != (unsigned)(nchunk - 1)) return false;
+  // last CTA: every other chunk's partial sums are in memory.  All threads add them, GT / V per
+  // value, then a tree over those (one thread per value walking the chunks took up to 50 us)
+  __threadfence();
+  constexpr int parts = GT / V;
+  const double *src = partial + threadIdx.x % V;
+  double v = 0.0;
+#pragma unroll 4
+  for (int cc = threadIdx.x / V; cc < nchunk; cc += parts) v += __ldcg(src + (long long)cc * V);
+  tot[threadIdx.x] = v;
+  for (int o = parts / 2; o > 0; o >>= 1) {
+    __syncthreads();
+    if (threadIdx.x < o * V) tot[threadIdx.x] += tot[threadIdx.x + o * V];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *count = 0u;
+  return true;
+}
+
 template <typename T, int BP, int BQ>
 __global__ void __launch_bounds__(GT)
 k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
@@ -146,41 +187,9 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
 #pragma unroll
       for (int j = 0; j < BQ; ++j) acc[i * BQ + j] = fma(a[i], b[j], acc[i * BQ + j]);
   }
-  warp_halving_sum<V>(acc);
-  __shared__ T red[GT / 32][V];
-  __shared__ unsigned ticket;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (halving_writer<V>(lane)) red[warp][halving_index<V>(lane)] = acc[0];
-  __syncthreads();
-  const long long blk = (long long)s * npb + pb;
-  if (threadIdx.x < V) {
-    T v = T(0);
-    for (int w = 0; w < GT / 32; ++w) v += red[w][threadIdx.x];
-    partial[(blk * nchunk + c) * V + threadIdx.x] = (double)v;
-    __threadfence();  // this chunk's sums are visible before the ticket is taken
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) ticket = atomicAdd(&count[blk], 1u);
-  __syncthreads();
-  if (ticket != (unsigned)(nchunk - 1)) return;
-  // last CTA of the block: every other chunk's partial sums are in memory.  All threads add
-  // them, GT / V per value, then a tree over those (one thread per value walking the chunks
-  // took up to 50 us)
-  __threadfence();
   __shared__ double tot[GT];
-  constexpr int parts = GT / V;
-  {
-    const double *src = partial + blk * nchunk * V + threadIdx.x % V;
-    double v = 0.0;
-#pragma unroll 4
-    for (int cc = threadIdx.x / V; cc < nchunk; cc += parts) v += __ldcg(src + (long long)cc * V);
-    tot[threadIdx.x] = v;
-  }
-  for (int o = parts / 2; o > 0; o >>= 1) {
-    __syncthreads();
-    if (threadIdx.x < o * V) tot[threadIdx.x] += tot[threadIdx.x + o * V];
-  }
-  __syncthreads();
+  const long long blk = (long long)s * npb + pb;
+  if (!chunk_sums<T, V>(acc, partial + blk * nchunk * V, count + blk, c, nchunk, tot)) return;
   if (threadIdx.x < V) {
     const double v = tot[threadIdx.x];
     const int i = i0 + threadIdx.x / BQ, j = j0 + threadIdx.x % BQ;
@@ -191,7 +200,6 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
         G[s * bsg + (long long)j * ldg + i] = v;
     }
   }
-  if (threadIdx.x == 0) count[blk] = 0u;  // re-armed for the next call on this stream
 }
 
 // Chunks of rows per block: two CTAs per SM in all, four for FP32 products, which wait for
@@ -287,6 +295,77 @@ k_update(const double *__restrict__ A, long long lda, long long bsa, int p,
         if (v1) dst[r1] = (beta == 0.0) ? x1 : fma(beta, dst[r1], x1);
       }
     }
+  }
+}
+
+// -------------------------- Arnoldi update and product ------------------------
+// C_s -= A_s y_s and, in the same pass over A, G_s = A_s^T C_s of the new C (GRAM: the second
+// classical Gram-Schmidt pass's coefficients) or G_s[0] = |C_s|^2 of it (the norm after the last
+// pass).  p <= BP columns, FP32 products and sums on the FP64 data, the norm in FP64.  Bound by
+// memory: A is read once where an update and a product after it read it twice.  INT: every other
+// column is converted by integer instructions, so that neither they nor the FP64 pipe, where
+// the hardware conversions run, take longer than the memory.
+template <int BP, bool GRAM, bool INT>
+__global__ void __launch_bounds__(GT)
+k_update_then(const double *__restrict__ A, long long lda, long long bsa, int p,
+              const double *__restrict__ Y, long long bsy, double *C, long long bsc,
+              long long nrows, int nchunk, double *__restrict__ partial,
+              unsigned *__restrict__ count, double *__restrict__ G, long long bsg) {
+  pdl_entry();
+  const int c = blockIdx.x, s = blockIdx.y;
+  __shared__ float y[BP];
+  if (threadIdx.x < BP) y[threadIdx.x] = threadIdx.x < p ? (float)-Y[s * bsy + threadIdx.x] : 0.f;
+  __syncthreads();
+  const double *As = A + s * bsa;
+  double *Cs = C + s * bsc;
+  const long long step = (long long)nchunk * GT;
+  float acc[BP] = {};
+  double nrm[1] = {0.0};
+  auto one = [&](const double (&x)[BP], double old, double *dst) {
+    float a[BP], u = 0.f;
+#pragma unroll
+    for (int i = 0; i < BP; ++i) {
+      a[i] = INT && (i & 1) ? load_as<float, true>(x[i]) : (float)x[i];
+      u = fmaf(a[i], y[i], u);
+    }
+    const double w = old + as_f64<INT>(u);
+    *dst = w;
+    if constexpr (GRAM) {
+      const float wf = load_as<float, INT>(w);
+#pragma unroll
+      for (int i = 0; i < BP; ++i) acc[i] = fmaf(a[i], wf, acc[i]);
+    } else {
+      nrm[0] = fma(w, w, nrm[0]);
+    }
+  };
+  // two rows per iteration: all of their loads are issued before the first use
+  long long r = (long long)c * GT + threadIdx.x;
+  for (; r + step < nrows; r += 2 * step) {
+    double x0[BP], x1[BP];
+    const double w0 = Cs[r], w1 = Cs[r + step];
+#pragma unroll
+    for (int i = 0; i < BP; ++i) {
+      x0[i] = i < p ? As[i * lda + r] : 0.0;
+      x1[i] = i < p ? As[i * lda + r + step] : 0.0;
+    }
+    one(x0, w0, Cs + r);
+    one(x1, w1, Cs + r + step);
+  }
+  if (r < nrows) {
+    double x[BP];
+#pragma unroll
+    for (int i = 0; i < BP; ++i) x[i] = i < p ? As[i * lda + r] : 0.0;
+    one(x, Cs[r], Cs + r);
+  }
+  __shared__ double tot[GT];
+  if constexpr (GRAM) {
+    if (!chunk_sums<float, BP>(acc, partial + (long long)s * nchunk * BP, count + s, c, nchunk, tot))
+      return;
+    if (threadIdx.x < p) G[s * bsg + threadIdx.x] = tot[threadIdx.x];
+  } else {
+    if (!chunk_sums<double, 1>(nrm, partial + (long long)s * nchunk, count + s, c, nchunk, tot))
+      return;
+    if (threadIdx.x == 0) G[s * bsg] = tot[0];
   }
 }
 
@@ -686,6 +765,34 @@ void launch_gram(const double *A, long long lda, long long bsa, int p, const dou
             : (BP == 2 ? TPS_GRAM(2, 1)
                        : (BP == 4 ? TPS_GRAM(4, 1) : (BP == 8 ? TPS_GRAM(8, 1) : TPS_GRAM(16, 1))));
 #undef TPS_GRAM
+}
+
+bool update_then_supported(int p) { return p >= 1 && p <= 16; }
+
+void launch_update_then(const double *A, long long lda, long long bsa, int p, const double *Y,
+                        long long bsy, double *C, long long bsc, long long nrows, bool gram,
+                        double *G, long long bsg, int batch, GramScratch &scr, cudaStream_t s) {
+  if (batch <= 0 || nrows <= 0 || !update_then_supported(p)) return;
+  const bool ints = nrows >= (1 << 20);  // as for the updates
+  int nchunk = gram_chunks(nrows, batch, 1, true);
+  const long long cap = scr.capacity / (batch * 16LL);
+  if (nchunk > cap) nchunk = (int)(cap > 0 ? cap : 1);
+  const dim3 grid(nchunk, batch);
+  count_launch();
+#define TPS_THEN(bp, gr, in)                                                                     \
+  launch_pdl(k_update_then<bp, gr, in>, grid, GT, 0, s, A, lda, bsa, p, Y, bsy, C, bsc, nrows,   \
+             nchunk, scr.partial, scr.count, G, bsg)
+#define TPS_THENP(gr, in)                                                                        \
+  (p <= 1 ? TPS_THEN(1, gr, in)                                                                  \
+          : p <= 2 ? TPS_THEN(2, gr, in)                                                         \
+                   : p <= 4 ? TPS_THEN(4, gr, in)                                                \
+                            : p <= 8 ? TPS_THEN(8, gr, in) : TPS_THEN(16, gr, in))
+  if (gram)
+    ints ? TPS_THENP(true, true) : TPS_THENP(true, false);
+  else
+    ints ? TPS_THENP(false, true) : TPS_THENP(false, false);
+#undef TPS_THENP
+#undef TPS_THEN
 }
 
 // Resident CTAs per SM of the k_update variants (queried once): FP64, FP32 products with the

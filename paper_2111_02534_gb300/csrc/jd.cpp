@@ -417,6 +417,7 @@ int alloc_workspace(tps_ctx *ctx, long long N, int mmax, int b, int kmax, int st
   w->gm.scale = take(b);
   w->gm.y = take((long long)b * steps);
   w->gm.h = take((long long)b * (steps + 1));
+  w->gm.h2 = take((long long)b * (steps + 1));
   w->gm.nrm2 = take(b);
   w->keep = reinterpret_cast<int *>(take(bw));
   w->keep0 = reinterpret_cast<int *>(take(bw));
@@ -505,14 +506,27 @@ int correction_impl(tps_ctx *ctx, const DevOperator &op, const double *Qt, int n
     kt_inverse(c, Qt, nq, KQt, use_prec, shift, w.W, nsys, w.P, shift_dev);
     if (use_prec) *prec_applies += nsys;
     // Arnoldi, classical Gram-Schmidt twice, per system: h = Z_i^T p_i ; p_i -= Z_i h
-    for (int pass = 0; pass < 2; ++pass) {
-      tgram(Z, (long long)nsys * N, N, j + 1, w.P, N, N, 1, N, w.gm.h, sst + 1, sst + 1, nsys,
-            ctx->gscr, s, nullptr, w.corr_low);
-      tupdate(Z, (long long)nsys * N, N, j + 1, w.gm.h, sst + 1, sst + 1, 1, -1.0, 1.0, w.P, N,
-              N, N, nsys, s, nullptr, w.corr_low);
-      launch_hess_add(nsys, sst, j, w.gm.h, sst + 1, w.gm, s);
+    const long long zs = (long long)nsys * N;
+    if (w.corr_low && update_then_supported(j + 1)) {
+      // the first pass's update with the second's product, the second's with the norm: Z and p
+      // are read three times instead of four, p once less for the norm
+      tgram(Z, zs, N, j + 1, w.P, N, N, 1, N, w.gm.h, sst + 1, sst + 1, nsys, ctx->gscr, s, nullptr,
+            true);
+      launch_update_then(Z, zs, N, j + 1, w.gm.h, sst + 1, w.P, N, N, true, w.gm.h2, sst + 1, nsys,
+                         ctx->gscr, s);
+      launch_update_then(Z, zs, N, j + 1, w.gm.h2, sst + 1, w.P, N, N, false, w.gm.nrm2, 1, nsys,
+                         ctx->gscr, s);
+      launch_hess_add(nsys, sst, j, w.gm.h, w.gm.h2, sst + 1, w.gm, s);
+    } else {
+      for (int pass = 0; pass < 2; ++pass) {
+        tgram(Z, zs, N, j + 1, w.P, N, N, 1, N, w.gm.h, sst + 1, sst + 1, nsys, ctx->gscr, s,
+              nullptr, w.corr_low);
+        tupdate(Z, zs, N, j + 1, w.gm.h, sst + 1, sst + 1, 1, -1.0, 1.0, w.P, N, N, N, nsys, s,
+                nullptr, w.corr_low);
+        launch_hess_add(nsys, sst, j, w.gm.h, nullptr, sst + 1, w.gm, s);
+      }
+      col_norms2(c, w.P, nsys, w.gm.nrm2);
     }
-    col_norms2(c, w.P, nsys, w.gm.nrm2);
     launch_gmres_givens(nsys, sst, j, w.gm.nrm2, w.gm, inner_tol, s);
     launch_scale_cols(nsys, N, w.P, N, w.gm.scale, 0, Z + (long long)(j + 1) * nsys * N, N, s);
   }

@@ -28,14 +28,17 @@ __global__ void k_gmres_init(int nsys, int s, const double *nrm2, double *beta, 
   scale[i] = ok ? -1.0 / b : 0.0;  // z_0 = -Kt^-1 r / beta
 }
 
-__global__ void k_hess_add(int nsys, int s, int j, const double *h, int ldh, double *Hb,
-                           const int *done) {
+__global__ void k_hess_add(int nsys, int s, int j, const double *h, const double *h2, int ldh,
+                           double *Hb, const int *done) {
   pdl_entry();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = e / (j + 1), l = e % (j + 1);
   if (i >= nsys) return;
   if (done[i]) return;
-  Hb[(long long)i * (s + 1) * s + (long long)j * (s + 1) + l] += h[(long long)i * ldh + l];
+  const long long at = (long long)i * ldh + l;
+  double *H = Hb + (long long)i * (s + 1) * s + (long long)j * (s + 1) + l;
+  const double v = *H + h[at];
+  *H = h2 ? v + h2[at] : v;
 }
 
 __global__ void k_gmres_givens(int nsys, int s, int j, const double *nrm2, double *Hb,
@@ -169,10 +172,10 @@ void launch_gmres_init(int nsys, int s, const double *nrm2, GmresState &st, cuda
              st.mvalid,
                                            st.scale);
 }
-void launch_hess_add(int nsys, int s, int j, const double *h, int ldh, GmresState &st,
-                     cudaStream_t str) {
+void launch_hess_add(int nsys, int s, int j, const double *h, const double *h2, int ldh,
+                     GmresState &st, cudaStream_t str) {
   count_launch();
-  launch_pdl(k_hess_add, nb((long long)nsys * (j + 1)), 128, 0, str, nsys, s, j, h, ldh, st.Hb,
+  launch_pdl(k_hess_add, nb((long long)nsys * (j + 1)), 128, 0, str, nsys, s, j, h, h2, ldh, st.Hb,
              st.done);
 }
 void launch_gmres_givens(int nsys, int s, int j, const double *nrm2, GmresState &st, double tol,

@@ -14,14 +14,16 @@ struct GmresState {
   double *scale = nullptr;  // [nsys]
   double *y = nullptr;      // [nsys][s]
   double *h = nullptr;      // [nsys][s+1] one Arnoldi column
+  double *h2 = nullptr;     // [nsys][s+1] its second Gram-Schmidt pass
   double *nrm2 = nullptr;   // [nsys]
   int *done = nullptr;      // [nsys]
   int *mvalid = nullptr;    // [nsys]
 };
 
 void launch_gmres_init(int nsys, int s, const double *nrm2, GmresState &st, cudaStream_t str);
-void launch_hess_add(int nsys, int s, int j, const double *h, int ldh, GmresState &st,
-                     cudaStream_t str);
+// adds h, and h2 unless null, to Hessenberg column j
+void launch_hess_add(int nsys, int s, int j, const double *h, const double *h2, int ldh,
+                     GmresState &st, cudaStream_t str);
 void launch_gmres_givens(int nsys, int s, int j, const double *nrm2, GmresState &st, double tol,
                          cudaStream_t str);
 void launch_gmres_solve(int nsys, int s, GmresState &st, cudaStream_t str);

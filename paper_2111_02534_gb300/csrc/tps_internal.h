@@ -127,6 +127,12 @@ void launch_update(const double *A, long long lda, long long bsa, int p, const d
                    long long bsy, int q, double alpha, double beta, double *C, long long ldc,
                    long long bsc, long long nrows, int batch, cudaStream_t s,
                    const int *need = nullptr, bool low = false);
+// C_s -= A_s y_s (p <= 16 columns, one column C_s per system) and in the same pass G_s = A_s^T C_s
+// (gram) or G_s[0] = |C_s|^2 of the new C_s; FP32 products on the FP64 data, the norm in FP64.
+bool update_then_supported(int p);
+void launch_update_then(const double *A, long long lda, long long bsa, int p, const double *Y,
+                        long long bsy, double *C, long long bsc, long long nrows, bool gram,
+                        double *G, long long bsg, int batch, GramScratch &scr, cudaStream_t s);
 // The same update, FP64-accurate, as digit-split BF16 products on the tensor cores
 // (update_mma.cu); q any, p any (slabs of 64).
 void launch_update_split(const double *A, long long lda, long long bsa, int p, const double *Y,
