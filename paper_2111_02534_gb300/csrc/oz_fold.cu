@@ -381,7 +381,6 @@ k_fold_gemm(const __grid_constant__ GemmArgs g) {
   uint32_t *holder = reinterpret_cast<uint32_t *>(drained + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    pdl_trigger();
     for (int i = 0; i < kStages; ++i) {
       tc::mbar_init(&full[i], 1);
       tc::mbar_init(&empty[i], 1);
@@ -396,6 +395,8 @@ k_fold_gemm(const __grid_constant__ GemmArgs g) {
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  // only now: a dependent kernel's CTA must not take tensor memory that this one waits for
+  if (threadIdx.x == 0) pdl_trigger();
   const uint32_t tmem = *holder;
   pdl_wait();
 

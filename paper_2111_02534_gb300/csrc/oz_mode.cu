@@ -34,10 +34,8 @@
 // same 16-byte column of consecutive rows writes consecutive addresses: no bank conflicts, no
 // padding of K beyond a multiple of 16.
 //
-// Digits: base 256, seven of a 55-bit integer for psi, eight of a 62-bit one for K, in FP16
-// (integers up to 2048 are exact).  q + 128 (1 + 256 + .. ) has the digits plus 128 as its
-// bytes, so a digit of two neighbours is one byte permute, one OR with FP16 1024 (whose unit is
-// 1) and one packed subtraction of 1152.
+// Digits (split_digits.cuh): base 256 in FP16, seven of a 55-bit integer for psi, eight of a
+// 62-bit one for K.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -89,7 +87,7 @@ struct Args {
   int *err;
   long long tiles;
   unsigned tm;   // tiles per vector
-  int w1, w9, w17, w25;  // 2, 2^9, 2^17, 2^25 (see level_sum)
+  b256::LevelWeights weights;
 };
 
 // Shared-memory matrix descriptor, K-major, no swizzle: bits 0-13 start address >> 4, bits
@@ -116,77 +114,6 @@ __device__ __forceinline__ void st4(double *p, const double (&v)[4]) {
                : "memory");
 }
 
-// round(x 2^(55 - E)) + 128 (1 + 2^8 + .. + 2^48), E = raw_max - 1022 (|x| < 2^E), mxe =
-// raw_max << 20: bytes 0 .. 5 are the lower six digits plus 128, the bits from 48 on the top
-// digit plus 128 (0 .. 256).  Subnormals count as zero.
-__device__ __forceinline__ uint64_t biased55(double x, unsigned mxe) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned exe = hi & 0x7FF00000u;
-  const unsigned sh = exe ? min((mxe - exe) >> 20, 63u) : 63u;
-  // the mantissa times 8 (56 bits), shifted right; with s = 0 or -1 the sign,
-  // (a ^ s) + 2 bias + 1 halved is bias +- round(a / 2), halves away from zero
-  const uint64_t m =
-      ((uint64_t)((((hi & 0xFFFFFu) | 0x100000u) << 3) | (lo >> 29)) << 32) | (lo << 3);
-  const uint64_t a = m >> sh;
-  const uint64_t s = (uint64_t)(long long)((int)hi >> 31);
-  return ((a ^ s) + 0x0101010101010101ULL) >> 1;
-}
-
-// The seven digits of two neighbouring elements as FP16 pairs, most significant first.
-__device__ __forceinline__ void digit_pairs(uint64_t u0, uint64_t u1, uint32_t (&d)[kSA]) {
-  const uint32_t l0 = (uint32_t)u0, h0 = (uint32_t)(u0 >> 32);
-  const uint32_t l1 = (uint32_t)u1, h1 = (uint32_t)(u1 >> 32);
-  const __half2 off = __half2half2(__ushort_as_half(0x6480));  // 1152
-  uint32_t w[kSA];
-  w[0] = __byte_perm(h0, h1, 0x7632) | 0x64006400u;
-  w[1] = (__byte_perm(h0, h1, 0x5511) & 0x00FF00FFu) | 0x64006400u;
-  w[2] = (__byte_perm(h0, h1, 0x5410) & 0x00FF00FFu) | 0x64006400u;
-  w[3] = (__byte_perm(l0, l1, 0x7733) & 0x00FF00FFu) | 0x64006400u;
-  w[4] = (__byte_perm(l0, l1, 0x7632) & 0x00FF00FFu) | 0x64006400u;
-  w[5] = (__byte_perm(l0, l1, 0x5511) & 0x00FF00FFu) | 0x64006400u;
-  w[6] = (__byte_perm(l0, l1, 0x5410) & 0x00FF00FFu) | 0x64006400u;
-#pragma unroll
-  for (int i = 0; i < kSA; ++i) {
-    const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&w[i]), off);
-    d[i] = *reinterpret_cast<const uint32_t *>(&h);
-  }
-}
-
-// sum_l d_l 2^(104 - 8 l) 2^(E - 117) rounded to FP64, E the sum of the two exponents.  As
-// sum_i |K[j][i]| < 2^(exponent of row j) the sum is below 2^E, so the levels add up modulo
-// 2^64 to its integer in units of 2^(E - 62); of level 7 (unit 2^(E - 69)) the part below is
-// rounded away, a quarter of what the digit pairs that are not kept weigh (2^(E - 60.5), root
-// mean square at 48 points).  One conversion on the FP64 pipe, otherwise idle here, rounds the
-// integer (a warp instruction takes that pipe ~64 cycles: about one per output is what fits
-// under the integer work; rounding by integer instructions costs ~20 more of them).  The
-// powers of two come from the kernel's arguments: as constants they would become shifts and
-// adds on the ALU, the busiest pipe, where the multiply-adds run on the FMA pipe.
-__device__ __forceinline__ double level_sum(const int (&d)[kL], int E, const Args &g) {
-  const int t7 = (d[7] + 64) >> 7;
-  long long t;
-  asm("{\n\t.reg .b64 t;\n\t"
-      "cvt.s64.s32 t, %5;\n\t"
-      "mad.wide.s32 t, %4, %6, t;\n\t"
-      "mad.wide.s32 t, %3, %7, t;\n\t"
-      "mad.wide.s32 t, %2, %8, t;\n\t"
-      "mad.wide.s32 %0, %1, %9, t;\n\t}"
-      : "=l"(t)
-      : "r"(d[3]), "r"(d[4]), "r"(d[5]), "r"(d[6]), "r"(t7), "r"(g.w1), "r"(g.w9), "r"(g.w17),
-        "r"(g.w25));
-  const unsigned top = (unsigned)(d[0] * g.w17) + (unsigned)(d[1] * g.w9) +
-                       (unsigned)(d[2] * g.w1);
-  t = (long long)((unsigned long long)t + ((unsigned long long)top << 32));
-  const int e = E - 62;
-  if (e < -1000 || e > 900) {  // near the ends of the range: two factors
-    const int h = e / 2;
-    return (double)t * b256::pow2d(h) * b256::pow2d(e - h);
-  }
-  // times 2^e in the exponent field (1023 .. 1086 for a nonzero integer)
-  const double v = (double)t;
-  const int hi = __double2hiint(v);
-  return __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(v));
-}
-
 // The digit image of K (n x n, row-major): for every sub-tile of 16 rows of K, 128 rows (digit
 // j of row c at 16 j + c) x 16 KC points in the operand layout; zeros beyond n.  A row's
 // exponent is its absolute sum's (see level_sum).
@@ -208,25 +135,7 @@ __global__ void k_build_image(const double *__restrict__ K, int n, int kc,
     __half h[8];
     for (int e = 0; e < 8; ++e) {
       const int i = col * 8 + e;
-      int d = 0;
-      if (r < n && i < n && ex[r]) {
-        // digit j of the 62-bit integer of K[r][i]
-        const unsigned long long x =
-            (unsigned long long)__double_as_longlong(K[(long long)r * n + i]);
-        const int raw = (int)((x >> 52) & 0x7FF);
-        long long q = 0;
-        if (raw) {
-          const long long mant = (long long)((x & ((1ULL << 52) - 1)) | (1ULL << 52));
-          const int sh = raw - (int)ex[r] + 9;
-          if (sh >= 0)
-            q = mant << sh;
-          else if (sh > -63)
-            q = (mant + (1LL << (-sh - 1))) >> (-sh);
-          if (x >> 63) q = -q;
-        }
-        const unsigned long long u = (unsigned long long)q + 0x0080808080808080ULL;
-        d = j == 0 ? (int)((long long)u >> 56) : (int)((u >> (8 * (7 - j))) & 0xFF) - 128;
-      }
+      const int d = r < n && i < n && ex[r] ? b256::digit62(K[(long long)r * n + i], ex[r], j) : 0;
       h[e] = __int2half_rn(d);
     }
     image[p] = *reinterpret_cast<const uint4 *>(h);
@@ -257,7 +166,6 @@ k_mode_product(const __grid_constant__ Args g) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    pdl_trigger();
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&fullA[i], C::kProdWarps);
       tc::mbar_init(&emptyA[i], 1);
@@ -281,6 +189,8 @@ k_mode_product(const __grid_constant__ Args g) {
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  // only now: a dependent kernel's CTA must not take tensor memory that this one waits for
+  if (threadIdx.x == 0) pdl_trigger();
   const uint32_t tmem = *holder;
   // the operator's image above is older than the previous kernel; everything below is not
   pdl_wait();
@@ -366,8 +276,8 @@ k_mode_product(const __grid_constant__ Args g) {
           uint32_t d[2][kSA];
 #pragma unroll
           for (int j = 0; j < 2; ++j)
-            digit_pairs(biased55(x[4 * k + 2 * j], mx[k]), biased55(x[4 * k + 2 * j + 1], mx[k]),
-                        d[j]);
+            b256::digit_pairs(b256::biased55(x[4 * k + 2 * j], mx[k]),
+                              b256::biased55(x[4 * k + 2 * j + 1], mx[k]), d[j]);
 #pragma unroll
           for (int i = 0; i < kSA; ++i)
             *reinterpret_cast<uint2 *>(dst + i * C::kSlice + 8 * k * 16) =
@@ -379,7 +289,7 @@ k_mode_product(const __grid_constant__ Args g) {
           uint32_t d[4][kSA];
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            digit_pairs(biased55(x[c * 8 + 2 * k], mx[0]), biased55(x[c * 8 + 2 * k + 1], mx[0]),
+            b256::digit_pairs(b256::biased55(x[c * 8 + 2 * k], mx[0]), b256::biased55(x[c * 8 + 2 * k + 1], mx[0]),
                         d[k]);
 #pragma unroll
           for (int i = 0; i < kSA; ++i)
@@ -439,7 +349,7 @@ k_mode_product(const __grid_constant__ Args g) {
             int d[kL];
 #pragma unroll
             for (int l = 0; l < kL; ++l) d[l] = __float2int_rn(__uint_as_float(rr[l][q]));
-            val[q] = level_sum(d, Em + sEn[c0 + h + q], g);
+            val[q] = b256::level_sum(d, Em + sEn[c0 + h + q], g.weights);
           }
           const unsigned c = c0 + h;
           if (valid) {
@@ -625,10 +535,7 @@ cudaError_t launch_mode_product(const ModeArgs &a, cudaStream_t s) {
   g.err = a.err;
   g.tm = (unsigned)((M + kRows - 1) / kRows);
   g.tiles = (long long)g.tm * a.nvec;
-  g.w1 = 1 << 1;
-  g.w9 = 1 << 9;
-  g.w17 = 1 << 17;
-  g.w25 = 1 << 25;
+  g.weights = b256::level_weights();
   const uintptr_t al = reinterpret_cast<uintptr_t>(a.psi) | reinterpret_cast<uintptr_t>(a.out);
   const bool vec = a.sigma == 1 && a.n % 4 == 0 && (al & 31) == 0;
   const Epi epi = !a.store ? kAdd : vec ? kStoreVec : kStore;

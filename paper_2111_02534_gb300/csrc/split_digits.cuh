@@ -1,20 +1,32 @@
-// Digit arithmetic of the FP64-accurate split products (block updates): the row-scaled
-// 54-bit integer of an FP64 value cut into seven base-256 digits, and the exact rounding of
-// the recombined levels back to FP64.  Shared by the tensor-core update kernels.
+// Digit arithmetic of the FP64-accurate split products (block updates, Gram products, the fused
+// 2D mode product): the scaled integer of an FP64 value cut into base-256 digits, and the exact
+// rounding of the recombined levels back to FP64.  Two cuts of the same 55-bit integer:
 //
-// Digits: a = |x| 2^(55 - E) truncated to an integer, E the row exponent (|x| < 2^E), so
-// a < 2^55, written as a = t 2^48 + c1 2^24 + c2 (t <= 127, c < 2^24), each 24-bit chunk
-// c = d0 2^16 + d1 2^8 + d2 with d0 in [0, 256] and |d1|, |d2| <= 128 (two FP32 roundings,
-// exact), the sign of x applied to every digit.  Integers up to 256 are exact in BF16; digit
-// i weighs 2^(E - 7 - 8 i).  The truncation error is below 2^-55 of the row maximum.
+//  * digits_pair (BF16; block updates and Gram products, mma.sync):
+//    Digits: a = |x| 2^(55 - E) truncated to an integer, E the row exponent (|x| < 2^E), so
+//    a < 2^55, written as a = t 2^48 + c1 2^24 + c2 (t <= 127, c < 2^24), each 24-bit chunk
+//    c = d0 2^16 + d1 2^8 + d2 with d0 in [0, 256] and |d1|, |d2| <= 128 (two FP32 roundings,
+//    exact), the sign of x applied to every digit.  Integers up to 256 are exact in BF16; digit
+//    i weighs 2^(E - 7 - 8 i).  The truncation error is below 2^-55 of the row maximum.
 //
-// Exactness of the level sums: with these digit bounds the products d_i(A) d_j(Y) of one
-// level l = i + j add up to at most 196352 (l = 5; 163840 to 179968 for l = 6, 7) per
-// contraction index, so over p <= 64 indices every partial sum is an integer below 2^23.6,
-// exact in an FP32 accumulator.
+//    Exactness of the level sums: with these digit bounds the products d_i(A) d_j(Y) of one
+//    level l = i + j add up to at most 196352 (l = 5; 163840 to 179968 for l = 6, 7) per
+//    contraction index, so over p <= 64 indices every partial sum is an integer below 2^23.6,
+//    exact in an FP32 accumulator.
+//
+//  * digit_pairs (FP16; the fused mode product): q = x 2^(55 - E) rounded to an integer, |q| <=
+//    2^55, in seven balanced digits, |d| <= 128.  Integers up to 2048 are exact in FP16: q + 128
+//    (1 + 256 + .. ) has the digits plus 128 as its bytes, so a digit of two values is one byte
+//    permute, one OR with the FP16 number 1024 (whose unit is 1) and one packed subtraction of
+//    1152: fewer instructions (57 against about 70 for a pair of values) but nearly all on the
+//    ALU.  In the kernels whose other work is also there the first cut, which spreads over the
+//    FP32 and conversion units, is faster (Gram product of 16 and 8 columns of 5.3 M rows 428 us
+//    against 451; update of 36 by 8 over 131,584 rows 28.1 against 28.7).
+//    The products of one level are at most 7 2^14 per index, below 2^23 over 64.
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <cstdint>
 
@@ -128,6 +140,100 @@ __device__ __forceinline__ void digits7(double x, unsigned raw_max, float (&d)[k
     d[2 + 3 * h] = d1;
     d[3 + 3 * h] = fmaf(-d1, 256.f, f);
   }
+}
+
+// round(x 2^(55 - E)) + 128 (1 + 2^8 + .. + 2^48), E = raw_max - 1022 (|x| < 2^E), mxe =
+// raw_max << 20: bytes 0 .. 5 are the lower six digits plus 128, the bits from 48 on the top
+// digit plus 128 (0 .. 256).  Subnormals count as zero.
+__device__ __forceinline__ uint64_t biased55(double x, unsigned mxe) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned exe = hi & 0x7FF00000u;
+  const unsigned sh = exe ? min((mxe - exe) >> 20, 63u) : 63u;
+  // the mantissa times 8 (56 bits), shifted right; with s = 0 or -1 the sign,
+  // (a ^ s) + 2 bias + 1 halved is bias +- round(a / 2), halves away from zero
+  const uint64_t m =
+      ((uint64_t)((((hi & 0xFFFFFu) | 0x100000u) << 3) | (lo >> 29)) << 32) | (lo << 3);
+  const uint64_t a = m >> sh;
+  const uint64_t s = (uint64_t)(long long)((int)hi >> 31);
+  return ((a ^ s) + 0x0101010101010101ULL) >> 1;
+}
+
+// The seven digits of two neighbouring elements as FP16 pairs, most significant first.
+__device__ __forceinline__ void digit_pairs(uint64_t u0, uint64_t u1, uint32_t (&d)[kUS]) {
+  const uint32_t l0 = (uint32_t)u0, h0 = (uint32_t)(u0 >> 32);
+  const uint32_t l1 = (uint32_t)u1, h1 = (uint32_t)(u1 >> 32);
+  const __half2 off = __half2half2(__ushort_as_half(0x6480));  // 1152
+  uint32_t w[kUS];
+  w[0] = __byte_perm(h0, h1, 0x7632) | 0x64006400u;
+  w[1] = (__byte_perm(h0, h1, 0x5511) & 0x00FF00FFu) | 0x64006400u;
+  w[2] = (__byte_perm(h0, h1, 0x5410) & 0x00FF00FFu) | 0x64006400u;
+  w[3] = (__byte_perm(l0, l1, 0x7733) & 0x00FF00FFu) | 0x64006400u;
+  w[4] = (__byte_perm(l0, l1, 0x7632) & 0x00FF00FFu) | 0x64006400u;
+  w[5] = (__byte_perm(l0, l1, 0x5511) & 0x00FF00FFu) | 0x64006400u;
+  w[6] = (__byte_perm(l0, l1, 0x5410) & 0x00FF00FFu) | 0x64006400u;
+#pragma unroll
+  for (int i = 0; i < kUS; ++i) {
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&w[i]), off);
+    d[i] = *reinterpret_cast<const uint32_t *>(&h);
+  }
+}
+
+// Digit j of the 62-bit integer round(x 2^(62 - E)), E = raw_max - 1022, in eight digits.
+__device__ __forceinline__ int digit62(double x, unsigned raw_max, int j) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int raw = (int)((b >> 52) & 0x7FF);
+  long long q = 0;
+  if (raw) {
+    const long long mant = (long long)((b & ((1ULL << 52) - 1)) | (1ULL << 52));
+    const int sh = raw - (int)raw_max + 9;
+    if (sh >= 0)
+      q = mant << sh;
+    else if (sh > -63)
+      q = (mant + (1LL << (-sh - 1))) >> (-sh);
+    if (b >> 63) q = -q;
+  }
+  const unsigned long long u = (unsigned long long)q + 0x8080808080808080ULL;
+  return (int)((u >> (8 * (7 - j))) & 0xFF) - 128;
+}
+
+// sum_l d_l 2^(104 - 8 l) 2^(E - 117) rounded to FP64: the levels of seven digits of A (scale
+// 2^E_A) times eight digits of B, the scale 2^E_B of a column of B being its absolute sum, E =
+// E_A + E_B.  As the sum is then below 2^E, the levels add up modulo 2^64 to its integer in
+// units of 2^(E - 62); of level 7 (unit 2^(E - 69)) the part below is rounded away, a quarter of
+// what the digit pairs that are not kept weigh (2^(E - 60.5), root mean square at 48 indices).
+// One conversion on the FP64 pipe rounds the integer (a warp instruction takes that pipe ~64
+// cycles; rounding by integer instructions costs ~20 more of them).  w1, w9, w17, w25 = 2, 2^9,
+// 2^17, 2^25 come from the kernel's arguments or constant memory: as immediates they would become
+// shifts and adds on the ALU, the busiest pipe, where the multiply-adds run on the FMA pipe.
+struct LevelWeights {
+  int w1, w9, w17, w25;
+};
+inline LevelWeights level_weights() { return {1 << 1, 1 << 9, 1 << 17, 1 << 25}; }
+__device__ __forceinline__ double pow2d(int e);
+__device__ __forceinline__ double level_sum(const int (&d)[kUL], int E, const LevelWeights &g) {
+  const int t7 = (d[7] + 64) >> 7;
+  long long t;
+  asm("{\n\t.reg .b64 t;\n\t"
+      "cvt.s64.s32 t, %5;\n\t"
+      "mad.wide.s32 t, %4, %6, t;\n\t"
+      "mad.wide.s32 t, %3, %7, t;\n\t"
+      "mad.wide.s32 t, %2, %8, t;\n\t"
+      "mad.wide.s32 %0, %1, %9, t;\n\t}"
+      : "=l"(t)
+      : "r"(d[3]), "r"(d[4]), "r"(d[5]), "r"(d[6]), "r"(t7), "r"(g.w1), "r"(g.w9), "r"(g.w17),
+        "r"(g.w25));
+  const unsigned top = (unsigned)(d[0] * g.w17) + (unsigned)(d[1] * g.w9) +
+                       (unsigned)(d[2] * g.w1);
+  t = (long long)((unsigned long long)t + ((unsigned long long)top << 32));
+  const int e = E - 62;
+  if (e < -1000 || e > 900) {  // near the ends of the range: two factors
+    const int h = e / 2;
+    return (double)t * pow2d(h) * pow2d(e - h);
+  }
+  // times 2^e in the exponent field (1023 .. 1086 for a nonzero integer)
+  const double v = (double)t;
+  const int hi = __double2hiint(v);
+  return __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(v));
 }
 
 __device__ __forceinline__ double pow2d(int e) {

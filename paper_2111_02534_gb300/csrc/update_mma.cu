@@ -6,14 +6,16 @@
 // The products are emulated by error-free digit splitting (the Ozaki scheme: Ozaki,
 // Ogita, Oishi & Rump, Numer. Algorithms 59, 2012), as in the H-apply, with digits sized
 // for a contraction of at most 64 terms (split_digits.cuh):
-//  * row r of A gets the exponent E_r with |A[r][k]| < 2^E_r for all k, column j of
-//    alpha Y the exponent F_j; each value becomes the integer |x| 2^(55 - E), truncated,
-//    written in seven signed base-256 digits, most significant first;
-//  * the digit pairs (i, j) with i + j <= 7 (34 of the 49) are multiplied in BF16 and the
-//    pairs of one level l = i + j are summed in one FP32 accumulator, exactly (every
-//    partial sum is an integer below 2^23.6 for p <= 64);
-//  * the levels are combined in two int64 Horner sums (levels 0-3 and 4-7) and rounded
-//    once to FP64 by integer arithmetic.
+//  * row r of A gets the exponent E_r with |A[r][k]| < 2^E_r for all k, column j of alpha Y the
+//    exponent F_j of its largest entry (p <= 16: of its absolute sum); each value becomes the
+//    integer |x| 2^(55 - E), truncated, written in seven signed base-256 digits, most
+//    significant first (p <= 16: alpha Y's x 2^(62 - F), rounded, in eight balanced ones);
+//  * the digit pairs (i, j) with i + j <= 7 (34 or 35) are multiplied in BF16 and the pairs of
+//    one level l = i + j are summed in one FP32 accumulator, exactly (every partial sum is an
+//    integer below 2^23.6 for p <= 64);
+//  * the levels are combined in two int64 Horner sums (levels 0-3 and 4-7) and rounded once to
+//    FP64 by integer arithmetic; for p <= 16 they add up in one 64-bit integer, which the FP64
+//    pipe rounds (p = 16, q = 3, 5.3 M rows: 438 -> 360 us).
 // The dropped levels l >= 8 weigh at most 131072 p 2^(E_r + F_j - 78) < p 2^-61 2^(E_r +
 // F_j) per entry, and the truncation of the operands to 55 bits 2^-55 of the row maximum:
 // the result has the accuracy of an FP64 product, 2^-53 max_k |A[r][k]| sum_k |alpha Y[k][j]|
@@ -54,6 +56,10 @@ namespace {
 
 using namespace b256;
 constexpr int kUKT = 4;         // k tiles of 16 (p <= 64)
+// Digits of alpha Y and the way the levels are put together, by the k tiles: with one (p <= 16)
+// the outputs are many for their digits, and the 64-bit sum pays (see the top); with more it
+// costs a digit pair per k (p = 36, q = 8 over 131,584 rows: 28.7 us against 28.1).
+__host__ __device__ constexpr int y_digits(int KT) { return KT == 1 ? 8 : kUS; }
 constexpr int kWarps = 8;       // consumer warps, 16 rows each
 constexpr int kCons = 32 * kWarps;
 constexpr int kRows = 16 * kWarps;  // rows per staged tile
@@ -109,6 +115,7 @@ struct UpdArgs {
   int stages;     // staged kernel: ring stages
   bool has_beta;  // beta != 0: C is read
 };
+__constant__ LevelWeights kWeights = {1 << 1, 1 << 9, 1 << 17, 1 << 25};
 
 // One warp: 16 rows (ra = row0 + g, rb = ra + 8) of C's columns j0 .. j0 + 7, with A's
 // entry (k, row r of the block) at As[k * cs + r] (r < 16, rows past nrows not read), KT
@@ -119,7 +126,7 @@ struct UpdArgs {
 // warp has read its last value of As.
 template <int KT, int NG, typename Stride, typename Release>
 __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Stride cs,
-                                        long long row0, const uint2 (*Bd)[kUS][kUKT][32],
+                                        long long row0, const uint2 (*Bd)[y_digits(KT)][kUKT][32],
                                         const unsigned (*Fraw)[8], int j0, double *Cs,
                                         Release release) {
   const int lane = threadIdx.x & 31;
@@ -181,7 +188,7 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
     for (int gg = 0; gg < NG; ++gg) {
       if (full16) {
 #pragma unroll
-        for (int j = 0; j < kUS; ++j) {
+        for (int j = 0; j < y_digits(KT); ++j) {
           const uint2 b = Bd[gg][j][kt][lane];
 #pragma unroll
           for (int i = 0; i < kUS; ++i)
@@ -189,7 +196,7 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < kUS; ++j) {
+        for (int j = 0; j < y_digits(KT); ++j) {
           const uint32_t b = Bd[gg][j][kt][lane].x;
 #pragma unroll
           for (int i = 0; i < kUS; ++i)
@@ -198,8 +205,7 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
       }
     }
   }
-  // combine the levels: value = (hi 2^32 + lo) 2^(E + F - 70), hi = levels 0..3, lo =
-  // levels 4..7 (Horner in base 256)
+  // combine the levels
 #pragma unroll
   for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
@@ -208,18 +214,25 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
     const int jl = 2 * c + (t & 1);
     const int j = j0 + 8 * gg + jl;
     if (!v || j >= g_.q) continue;
-    long long hi = 0, lo = 0;
-#pragma unroll
-    for (int l = 0; l < kUL; ++l) {
-      const long long dl = (long long)__float2int_rn(acc[gg][l][t]);
-      if (l < kUL / 2)
-        hi = hi * 256 + dl;
-      else
-        lo = lo * 256 + dl;
-    }
     const unsigned er = (t & 2) ? eb : ea, fr = Fraw[gg][jl];
-    const double val =
-        (er && fr) ? combine(hi, lo, (int)er - 1022 + (int)fr - 1022) : 0.0;
+    double val = 0.0;
+    if constexpr (y_digits(KT) == 8) {
+      int d[kUL];
+#pragma unroll
+      for (int l = 0; l < kUL; ++l) d[l] = __float2int_rn(acc[gg][l][t]);
+      if (er && fr) val = level_sum(d, (int)er - 1022 + (int)fr - 1022, kWeights);
+    } else {  // (hi 2^32 + lo) 2^(E - 70): Horner sums in base 256 of levels 0-3 and 4-7
+      long long hi = 0, lo = 0;
+#pragma unroll
+      for (int l = 0; l < kUL; ++l) {
+        const long long dl = (long long)__float2int_rn(acc[gg][l][t]);
+        if (l < kUL / 2)
+          hi = hi * 256 + dl;
+        else
+          lo = lo * 256 + dl;
+      }
+      if (er && fr) val = combine(hi, lo, (int)er - 1022 + (int)fr - 1022);
+    }
     double *dst = Cs + (long long)j * g_.ldc + ((t & 2) ? rb : ra);
     *dst = g_.has_beta ? fma(g_.beta, *dst, val) : val;
   }
@@ -227,33 +240,52 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
 
 // Digit planes of alpha Y's columns j0 .. j0 + 7 as m16n8k16 B fragments in shared memory,
 // and their column exponents; the kCons consumer threads take part.
+template <int YS>
 __device__ __forceinline__ void y_fragments(const UpdArgs &g_, const double *Ys, int j0,
                                             uint2 (*Bd)[kUKT][32], unsigned *Fraw) {
+  // a column's scale is the exponent of its absolute sum for eight digits (see level_sum), of
+  // its largest entry for seven
   const int t = threadIdx.x;
   if (t < 128) {
     const int jl = t >> 4, k0 = t & 15, j = j0 + jl;
     unsigned m = 0;
-    if (j < g_.q)
+    if constexpr (YS == 8) {
+      double sum = 0.0;
+      if (j < g_.q)
 #pragma unroll
-      for (int k = k0; k < 64; k += 16)
-        if (k < g_.p) m = max(m, raw_exp(g_.alpha * Ys[(long long)j * g_.ldy + k]));
+        for (int k = k0; k < 64; k += 16)
+          if (k < g_.p) sum += fabs(g_.alpha * Ys[(long long)j * g_.ldy + k]);
 #pragma unroll
-    for (int o = 1; o < 16; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      for (int o = 1; o < 16; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      m = raw_exp(sum);
+    } else {
+      if (j < g_.q)
+#pragma unroll
+        for (int k = k0; k < 64; k += 16)
+          if (k < g_.p) m = max(m, raw_exp(g_.alpha * Ys[(long long)j * g_.ldy + k]));
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    }
     if (k0 == 0) Fraw[jl] = m;
   }
   asm volatile("bar.sync 1, %0;" ::"r"(kCons) : "memory");
   if (t < 32 * kUKT) {
     const int kt = t >> 5, lane = t & 31, g = lane >> 2, c = lane & 3;
     const int j = j0 + g;
-    float dv[4][kUS];
+    float dv[4][YS];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int k = 16 * kt + 2 * c + (e & 1) + 8 * (e >> 1);
       const double y = (j < g_.q && k < g_.p) ? g_.alpha * Ys[(long long)j * g_.ldy + k] : 0.0;
-      digits7(y, Fraw[g], dv[e]);
+      if constexpr (YS == 8) {
+#pragma unroll
+        for (int i = 0; i < YS; ++i) dv[e][i] = (float)digit62(y, Fraw[g], i);
+      } else {
+        digits7(y, Fraw[g], dv[e]);
+      }
     }
 #pragma unroll
-    for (int i = 0; i < kUS; ++i)
+    for (int i = 0; i < YS; ++i)
       Bd[i][kt][lane] = make_uint2(pack_bf16(dv[0][i], dv[1][i]), pack_bf16(dv[2][i], dv[3][i]));
   }
   asm volatile("bar.sync 1, %0;" ::"r"(kCons) : "memory");
@@ -266,10 +298,10 @@ __global__ void __launch_bounds__(kCons)
 k_update_split(const __grid_constant__ UpdArgs g_) {
   pdl_entry();
   if (g_.need && *g_.need == 0) return;  // conditional product (decided on the device)
-  __shared__ uint2 Bd[1][kUS][kUKT][32];
+  __shared__ uint2 Bd[1][y_digits(KT)][kUKT][32];
   __shared__ unsigned Fraw[1][8];
   const int s = blockIdx.y, j0 = blockIdx.z * 8, warp = threadIdx.x >> 5;
-  y_fragments(g_, g_.Y + s * g_.bsy, j0, Bd[0], Fraw[0]);
+  y_fragments<y_digits(KT)>(g_, g_.Y + s * g_.bsy, j0, Bd[0], Fraw[0]);
   const double *As = g_.A + s * g_.bsa;
   double *Cs = g_.C + s * g_.bsc;
   const long long nblk = (g_.nrows + 15) >> 4;
@@ -288,7 +320,7 @@ k_update_split_staged(const __grid_constant__ UpdArgs g_) {
   pdl_entry();
   if (g_.need && *g_.need == 0) return;
   extern __shared__ __align__(128) double ring[];
-  __shared__ uint2 Bd[NG][kUS][kUKT][32];
+  __shared__ uint2 Bd[NG][y_digits(KT)][kUKT][32];
   __shared__ unsigned Fraw[NG][8];
   __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages];
   __shared__ int abort_flag;
@@ -353,7 +385,7 @@ k_update_split_staged(const __grid_constant__ UpdArgs g_) {
   }
   // ---- consumers
 #pragma unroll
-  for (int gg = 0; gg < NG; ++gg) y_fragments(g_, g_.Y + s * g_.bsy, j0 + 8 * gg, Bd[gg], Fraw[gg]);
+  for (int gg = 0; gg < NG; ++gg) y_fragments<y_digits(KT)>(g_, g_.Y + s * g_.bsy, j0 + 8 * gg, Bd[gg], Fraw[gg]);
   int it = 0;
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
     const int st = it % S;
