@@ -39,17 +39,16 @@ REL_TOL = 1e-10
 FP64_FLOP_PER_CLK_PER_SM = 4
 N_SM = 152
 SM_MAX_MHZ = 2070.0
-# digit-pair products of the tensor-core FP64 emulation (9 wave-function digits, 10
-# mode-matrix digits, levels i + j <= 9 kept): each one a BF16 MMA over the full product
-TC_PAIRS = 54
+# digit-pair products of the tensor-core FP64 emulation (eight base-256 digits of either
+# operand, levels i + j <= 7 kept): each one an FP16 MMA over the folded product
+TC_PAIRS = 36
 # DRAM bytes (read + write) per launch of each kernel, mean over the launches of one ncu
 # capture of the kernel on this workload; a kernel that changes after its capture is
 # removed from this table
 TRAFFIC_BYTES_PER_LAUNCH = {"k_tf32_gemm": 5.08e6}
 # the same for kernels whose launches cover a varying number of vectors: (bytes per launch,
-# bytes per vector), fitted to two captured launches of different width (k_oz_gemm: 6 and 4
-# vectors, 49.65 and 35.66 MB)
-TRAFFIC_AFFINE = {"k_oz_gemm": (7.68e6, 6.99e6)}
+# bytes per vector), fitted to captured launches of different widths (none at present)
+TRAFFIC_AFFINE = {}
 TF32_PER_BF16 = 1.1 / 2.25   # nominal dense tensor rates per GPU (TF32, BF16)
 # BF16 digit-pair products per FP64 multiply-add of the split block update
 SPLIT_UPDATE_PAIRS = 34
@@ -572,14 +571,18 @@ def run_ours(args):
     step_s = local_t
     nx_s, ny = w.n[0] // 2 + 1, w.n[1]
     fp64_per_vec = 2.0 * nx_s * ny * (nx_s + ny) + 3.0 * nx_s * ny
-    tc_per_vec = 2.0 * TC_PAIRS * nx_s * ny * (nx_s + ny)
+    # multiply-adds of the folded products per line: the squares of the blocks' points (the
+    # periodic mode in four blocks, the sector's in two)
+    fold_y = (ny // 4 + 1) ** 2 + 3 * (ny // 4) ** 2
+    fold_x = ((nx_s + 1) // 2) ** 2 + (nx_s // 2) ** 2
+    tc_per_vec = 2.0 * TC_PAIRS * (nx_s * fold_y + ny * fold_x)
     kernels = {}
     h_ms, h_fl = tot("h_ms"), tot("h_flops")
     if h_ms > 0:
         tflops = h_fl / fp64_per_vec * tc_per_vec / (h_ms / 1000.0) / 1e12
-        kernels["k_oz_gemm"] = {
-            "what": "FP64 H-apply on tcgen05 (BF16 digit products, exact FP32 levels; with its "
-                    "digit-splitting kernels)",
+        kernels["k_fold_gemm"] = {
+            "what": "FP64 H-apply on tcgen05 (products folded by the modes' symmetry, FP16 "
+                    "digits, exact FP32 levels; with its splitting and unfolding kernels)",
             "bound": "tensor", "achieved": tflops, "peak": bf16_peak, "unit": "TFLOP/s",
             "frac": tflops / bf16_peak if bf16_peak else None,
             "peak_note": "bf16_tflops_sustained of measured (cuBLAS bf16, seconds-long loop)",

@@ -59,8 +59,9 @@ enum { TPS_ANY = 0, TPS_X_EVEN = 1, TPS_X_ODD = 2 }; /* heavy-exchange sector (S
 enum { TPS_F64 = 0, TPS_F32 = 1, TPS_F64_TC = 2, TPS_TF32_TC = 3 };  /* arithmetic of apply calls
                                                                        (data stay FP64) */
 /* TPS_F64_TC: FP64-accurate mode products emulated on the BF16 tensor cores by error-free
- * splitting into digit slices per operand row (1D: 9 six-bit digits for the wave function,
- * 10 for the mode matrices; 2D, at most 128 points per mode: 7 and 8 eight-bit digits;
+ * splitting into digit slices per operand row (1D: 8 eight-bit digits of either operand,
+ * folded by the symmetry of the mode matrices, or 9 and 10 six-bit digits where the folded
+ * blocks are longer than 146 points; 2D, at most 128 points per mode: 7 and 8 eight-bit digits;
  * Ozaki scheme), exact FP32 accumulation per digit level, FP64 recombination; H-apply only.
  * TPS_TF32_TC: the preconditioner's mode products on the tensor cores with TF32 inputs
  * (10 explicit mantissa bits) and FP32 accumulation, ~2.5e-3 relative to the exact
@@ -174,7 +175,8 @@ int tps_get_info(const tps_ctx *ctx, long long *N, double *hnorm_est);
  * 2^-53 n of row max x column max per product, like FP64 arithmetic).  The first
  * TPS_F64_TC call on a context builds the operator's digit slices (a few MB) and a
  * slice workspace of up to 256 MB (2D: the four mode products one after the other, a
- * fiber-slice workspace of up to 1 GB; TPS_ERR_INVALID_ARG for more than 128 points in a
+ * fiber-slice workspace of up to 1 GB if a mode has more than 64 points;
+ * TPS_ERR_INVALID_ARG for more than 128 points in a
  * mode). */
 int tps_apply_h(tps_ctx *ctx, const void *psi_dev, void *out_dev, int nvec, double theta,
                 int dtype, cudaStream_t stream);
