@@ -18,7 +18,8 @@
 //   warps 0-11   load psi (a warp takes 16 points of 32 fibers, in registers), agree on the
 //                fibers' exponents and write the seven digit slices straight into the operand
 //                layout in shared memory (two stages; one for more than 48 points);
-//   warps 12-27  drain the accumulators, recombine the levels and store;
+//   warps 12-27  copy the operator's image, then drain the accumulators, recombine the levels
+//                and store;
 //   warp 28      issues the MMAs.
 // (Eight producer and eight epilogue warps, with twice the registers: 115 us per mode instead
 // of 100.)
@@ -161,8 +162,8 @@ k_mode_product(const __grid_constant__ Args g) {
   int *sEn = reinterpret_cast<int *>(sMax + 2 * KC * kRows);  // [KC * kCols]
   uint64_t *bars = reinterpret_cast<uint64_t *>(sEn + KC * kCols);
   uint64_t *fullA = bars, *emptyA = bars + 2, *accum = bars + 4, *accfree = accum + kAcc;
-  uint64_t *drained = accfree + kAcc;
-  uint32_t *holder = reinterpret_cast<uint32_t *>(drained + 1);
+  uint64_t *drained = accfree + kAcc, *image = drained + 1;
+  uint32_t *holder = reinterpret_cast<uint32_t *>(image + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -175,24 +176,18 @@ k_mode_product(const __grid_constant__ Args g) {
       tc::mbar_init(&accfree[i], C::kEpiWarps);
     }
     tc::mbar_init(drained, 1);
+    tc::mbar_init(image, C::kEpiWarps);
     abort_flag = 0;
     tc::fence_barrier_init();
   }
   if (warp == C::kMmaWarp) tc::tmem_alloc(holder, kTmemCols);
-  {
-    uint4 *dst = reinterpret_cast<uint4 *>(sB);
-    for (unsigned i = threadIdx.x; i < C::kB / 16; i += C::kThreads) dst[i] = g.image[i];
-    for (unsigned i = threadIdx.x; i < KC * kCols; i += C::kThreads)
-      sEn[i] = i < g.n ? (int)g.eK[i] - 1022 : 0;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
   // only now: a dependent kernel's CTA must not take tensor memory that this one waits for
   if (threadIdx.x == 0) pdl_trigger();
   const uint32_t tmem = *holder;
-  // the operator's image above is older than the previous kernel; everything below is not
+  // every global access follows: the previous kernel may be the one that built the image
   pdl_wait();
 
   if (warp < C::kProdWarps) {
@@ -308,6 +303,18 @@ k_mode_product(const __grid_constant__ Args g) {
     const int quarter = warp & 3, part = (warp - C::kProdWarps) >> 2;
     const unsigned row = 32 * quarter + lane;
     const uint32_t trow = tmem + ((uint32_t)(32 * quarter) << 16) + part * EC;
+    {  // the operator's image, while the producers load and cut the first tile
+      const unsigned first = threadIdx.x - 32 * C::kProdWarps, step = 32 * C::kEpiWarps;
+      uint4 *dst = reinterpret_cast<uint4 *>(sB);
+#pragma unroll 4
+      for (unsigned i = first; i < C::kB / 16; i += step) dst[i] = g.image[i];
+      for (unsigned i = first; i < KC * kCols; i += step)
+        sEn[i] = i < g.n ? (int)g.eK[i] - 1022 : 0;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(image);
+      asm volatile("bar.sync 5, %0;" ::"r"(step) : "memory");  // sEn, for these warps
+    }
     int it = 0;
     unsigned u = 0;  // sub-tile counter
     bool alive = true;
@@ -372,7 +379,7 @@ k_mode_product(const __grid_constant__ Args g) {
     }
   } else if (lane == 0) {
     // ---- MMA issuer
-    bool ok = true;
+    bool ok = tc::mbar_wait(image, 0, g.err, 8);
     int it = 0;
     unsigned u = 0;
     const uint32_t a0 = tc::smem_addr(sA), b0 = tc::smem_addr(sB);
