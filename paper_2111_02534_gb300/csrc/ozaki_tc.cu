@@ -467,7 +467,6 @@ __device__ __forceinline__ void oz_tile(const CUtensorMap *tmAp, const CUtensorM
   const int KB = (g.K + kBK - 1) / kBK;
 
   if (threadIdx.x == 0) {
-    pdl_trigger();
     for (int i = 0; i < kAStages; ++i) {
       tc::mbar_init(&fullA[i], 1);
       tc::mbar_init(&emptyA[i], 1);
@@ -486,6 +485,8 @@ __device__ __forceinline__ void oz_tile(const CUtensorMap *tmAp, const CUtensorM
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  // only now: a dependent kernel's CTA must not take tensor memory that this one waits for
+  if (threadIdx.x == 0) pdl_trigger();
   const uint32_t tmem = *holder;
   // the set-up above overlaps the previous kernel; every global access below follows it
   pdl_wait();

@@ -139,7 +139,6 @@ k_tf32_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   const int KB = (g.K + kBK - 1) / kBK;
 
   if (threadIdx.x == 0) {
-    pdl_trigger();
     for (int i = 0; i < kStages; ++i) {
       tc::mbar_init(&full[i], 1);
       tc::mbar_init(&empty[i], 1);
@@ -154,6 +153,8 @@ k_tf32_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  // only now: a dependent kernel's CTA must not take tensor memory that this one waits for
+  if (threadIdx.x == 0) pdl_trigger();
   const uint32_t tmem = *holder;
 
   if (warp == 0 && lane == 0) {

@@ -32,3 +32,25 @@ def test_the_fused_mode_product_reads_nothing_before_its_wait():
     for what in ("image", "eK", "psi", "out"):
         assert f"g.{what}" not in before, what
         assert f"g.{what}" in body[len(before):], what
+
+
+_ALLOCATING = [(os.path.basename(path), name) for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+               for name, body in _functions(os.path.basename(path)).items() if "tmem_alloc(" in body]
+
+
+def test_the_kernels_with_tensor_memory_are_found():
+    assert {name for _, name in _ALLOCATING} >= {"oz_tile", "k_oz_gemm1p", "k_mode_product",
+                                                 "k_fold_gemm", "k_tf32_gemm"}
+
+
+@pytest.mark.parametrize("source,name", _ALLOCATING)
+def test_dependents_start_after_the_tensor_memory_is_allocated(source, name):
+    # a dependent's CTA on the same SM could otherwise take the tensor memory first and then wait
+    # for this kernel, whose allocation would wait for that CTA: the one wait without a limit
+    body = _functions(source)[name]
+    if "pdl_trigger()" not in body:
+        return
+    alloc = body.index("tmem_alloc(")
+    held = body.index("__syncthreads()", alloc)
+    assert body.index("pdl_trigger()") > held
+    assert "pdl_entry()" not in body
