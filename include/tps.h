@@ -172,7 +172,8 @@ int tps_get_info(const tps_ctx *ctx, long long *N, double *hnorm_est);
  * device, [nvec][N] FP64, must not overlap.  dtype TPS_F64: FP64 arithmetic; TPS_F32:
  * FP32 arithmetic (error ~ n eps_32 ||H|| |psi|), the low-precision phase's operator;
  * TPS_F64_TC: FP64-accurate products on the tensor cores (error below
- * 2^-53 n of row max x column max per product, like FP64 arithmetic).  The first
+ * 2^-53 n of row max x column max per product, like FP64 arithmetic).  A vector's result
+ * has the same bits whatever nvec is and wherever in the block it stands.  The first
  * TPS_F64_TC call on a context builds the operator's digit slices (a few MB) and a
  * slice workspace of up to 256 MB (2D: the four mode products one after the other, a
  * fiber-slice workspace of up to 1 GB if a mode has more than 64 points;

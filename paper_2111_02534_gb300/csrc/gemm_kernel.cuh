@@ -53,6 +53,7 @@ struct GemmArgs {
   const void *lamM, *lamN, *lam2, *lam3;
   int n2, n3;
   double sigma;
+  int split;  // FP64: warps that share a product's K (k_gemm_direct); 0: k_gemm
   int tiles_m, tiles_n;
 };
 
@@ -205,17 +206,16 @@ k_gemm(const GemmArgs g) {
 // FP64 products without shared-memory tiles.  GB300's FP64 pipe takes a warp instruction per
 // ~64 cycles of a scheduler, so a warp's FMA leaves time for its loads to come from L1 and L2,
 // whatever their reuse; what matters is that every scheduler of every SM has warps with FMAs to
-// issue.  A CTA computes (32 / LC) R x LC outputs, R per lane of each of its 8 warps, which
-// split K between them (adjacent pieces, added in order at the end: 7 FP64 additions per
-// output).  H-apply, tiled -> direct: 64 x 64, 1 vector 79 -> 9 us (one 64-thread CTA of the
-// tiled kernel runs all of K on two schedulers); 128 x 128, 4 vectors 150 -> 37; 512 x 512, 8
-// vectors 3610 -> 3480, 0.97 of the pipe.
-constexpr int kDirectWarps = 8;
-template <int R, int LC>
-__global__ void __launch_bounds__(32 * kDirectWarps)
+// issue.  A CTA computes (32 / LC) R x LC outputs, R per lane of each of its KS warps, which
+// split K between them (adjacent pieces, added in order at the end: KS - 1 FP64 additions per
+// output; f64_split in gemm_f64.cu chooses KS).  H-apply, tiled -> direct with KS = 8: 64 x 64, 1
+// vector 79 -> 9 us (one 64-thread CTA of the tiled kernel runs all of K on two schedulers); 128 x
+// 128, 4 vectors 150 -> 37; 512 x 512, 8 vectors 3610 -> 3480, 0.97 of the pipe.
+template <int R, int LC, int KS>
+__global__ void __launch_bounds__(32 * KS)
 k_gemm_direct(const GemmArgs g) {
   constexpr int LR = 32 / LC;
-  __shared__ double red[kDirectWarps][R][32];
+  __shared__ double red[KS][R][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tiles = g.tiles_m * g.tiles_n;
   const long long z = blockIdx.x / tiles;
@@ -227,8 +227,8 @@ k_gemm_direct(const GemmArgs g) {
   for (int i = 0; i < R; ++i) acc[i] = 0.0;
   for (int ph = 0; ph < g.nphase; ++ph) {
     const int K = g.K[ph];
-    const int k0 = (int)((long long)K * warp / kDirectWarps);
-    const int k1 = (int)((long long)K * (warp + 1) / kDirectWarps);
+    const int k0 = (int)((long long)K * warp / KS);
+    const int k1 = (int)((long long)K * (warp + 1) / KS);
     const double *Bp = static_cast<const double *>(g.B[ph].p) + z * g.B[ph].bs + nc;
     const double *Ap[R];
 #pragma unroll
@@ -260,24 +260,37 @@ k_gemm_direct(const GemmArgs g) {
 #pragma unroll
   for (int i = 0; i < R; ++i) red[warp][i][lane] = acc[i];
   __syncthreads();
-  if (warp >= R) return;
-  double c = red[0][warp][lane];
-#pragma unroll
-  for (int w = 1; w < kDirectWarps; ++w) c += red[w][warp][lane];
-  const int m = m0 + LR * warp;
-  if (m >= g.M || n >= g.Nc) return;
+  if (n >= g.Nc) return;
   const double th = g.epi != EPI_HAPPLY ? 0.0 : g.theta ? g.theta[z / g.theta_div] : g.theta0;
-  finish_element<double, double>(g, z, m, n, c, th);
+  for (int i = warp; i < R; i += KS) {
+    double c = red[0][i][lane];
+#pragma unroll
+    for (int w = 1; w < KS; ++w) c += red[w][i][lane];
+    const int m = m0 + LR * i;
+    if (m < g.M) finish_element<double, double>(g, z, m, n, c, th);
+  }
 }
 
-template <int R, int LC>
+template <int R, int LC, int KS>
 void run_direct(GemmArgs g, cudaStream_t s) {
   g.tiles_m = (g.M + 32 / LC * R - 1) / (32 / LC * R);
   g.tiles_n = (g.Nc + LC - 1) / LC;
   const long long blocks = (long long)g.batch * g.tiles_m * g.tiles_n;
   if (blocks <= 0) return;
   count_launch();
-  k_gemm_direct<R, LC><<<(unsigned)blocks, 32 * kDirectWarps, 0, s>>>(g);
+  k_gemm_direct<R, LC, KS><<<(unsigned)blocks, 32 * KS, 0, s>>>(g);
+}
+
+// Fewer outputs per lane while that leaves CTAs for two per SM; 32 columns per warp where rows
+// are that long (24^4, 4 vectors: 328 us, 369 with 8, both with KS = 8).  The bits do not depend
+// on either.
+template <int KS>
+void run_direct(const GemmArgs &g, cudaStream_t s) {
+  const long long out = (long long)g.M * g.Nc * g.batch;
+  if (out <= 32 * 304) return run_direct<1, 8, KS>(g, s);
+  if (out <= 64 * 304) return run_direct<2, 8, KS>(g, s);
+  if (g.Nc < 256) return run_direct<4, 8, KS>(g, s);
+  run_direct<4, 32, KS>(g, s);
 }
 
 // Tile choice: minimise padded work plus a one-tile-per-SM imbalance allowance,
@@ -357,19 +370,8 @@ TileCache &tile_cache();
 template <typename Acc, typename TA, typename TB, typename TC>
 void gemm(GemmArgs g, cudaStream_t s) {
   if constexpr (sizeof(Acc) == 8) {
-    // Many outputs of a short K keep the tiled kernel: splitting K costs 7 additions per output
-    // (2D H-apply of 2 vectors at 48^4, 10.6 M outputs a launch: tiled 3.62 ms, direct 4.55; at
-    // 48^2 x 24^2, 2.7 M outputs, 1.04 and 0.93).  Otherwise direct, with fewer outputs per
-    // lane while that leaves CTAs for two per SM; 32 columns per warp where rows are that long
-    // (24^4, 4 vectors: 328 us, 369 with 8).
-    const long long out = (long long)g.M * g.Nc * g.batch;
-    const int K = g.K[0] + (g.nphase > 1 ? g.K[1] : 0);
-    if (out < (1LL << 22) || K > 128) {
-      if (out <= 32 * 304) return run_direct<1, 8>(g, s);
-      if (out <= 64 * 304) return run_direct<2, 8>(g, s);
-      if (g.Nc < 256) return run_direct<4, 8>(g, s);
-      return run_direct<4, 32>(g, s);
-    }
+    if (g.split == 8) return run_direct<8>(g, s);
+    if (g.split == 2) return run_direct<2>(g, s);
   }
   int tm, tn;
   pick_tiles(g, tm, tn);
@@ -456,11 +458,14 @@ inline GemmArgs right(const void *A, long long rows, int n, const void *B, void 
 
 // Right product in row chunks small enough for int row counts.
 template <typename Acc, typename TA, typename TB, typename TC>
-void right_chunked(const TA *A, long long rows, int n, const TB *B, TC *C, cudaStream_t s) {
+void right_chunked(const TA *A, long long rows, int n, const TB *B, TC *C, cudaStream_t s,
+                   int split = 0) {
   const long long chunk = 1LL << 24;
   for (long long r0 = 0; r0 < rows; r0 += chunk) {
     const long long r = rows - r0 < chunk ? rows - r0 : chunk;
-    gemm<Acc, TA, TB, TC>(right(A + r0 * n, r, n, B, C + r0 * n), s);
+    GemmArgs g = right(A + r0 * n, r, n, B, C + r0 * n);
+    g.split = split;
+    gemm<Acc, TA, TB, TC>(g, s);
   }
 }
 

@@ -386,3 +386,29 @@ def test_apply_h_1d_around_the_direct_kernels_limits(n, nvec):
     P = problem_1d(20.0, 1.0, 1.0, n, (20.0, 15.0), 1.0, 1.0)
     ctx = make_ctx_1d(20.0, 1.0, n, (20.0, 15.0), 1.0, 1.0)
     _check_h(P, ctx, nvec, 0.3, seed=5)
+
+
+@pytest.mark.parametrize("n,nvec", [((64, 64), 1100), ((12, 30), 7), ((12, 12, 12, 12), 8),
+                                    ((6, 6, 20, 20), 3), ((40, 40, 40, 40), 2),
+                                    ((32, 32, 32, 32), 5), ((36, 36, 24, 24), 6),
+                                    ((4, 4, 66, 66), 3)])
+def test_fp64_results_do_not_depend_on_the_number_of_vectors(n, nvec):
+    # every form of the FP64 products, with blocks on both sides of 2^22 outputs; the bits of the
+    # first and the last vector of a block against calls with that vector alone
+    require_gpu()
+    from paper_2111_02534_gb300 import tps
+    L = (8.0,) * len(n)
+    ctx = make_ctx_1d(20.0, 1.0, n, L, 1.0, 1.0) if len(n) == 2 else \
+        make_ctx_2d(20.0, 1.0, n, L, 2.0, 1.0)
+    N = ctx.info()[0]
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(nvec, N, generator=g, dtype=torch.float64, device="cuda")
+    block, one = torch.empty_like(x), torch.empty(1, N, dtype=torch.float64, device="cuda")
+    for apply in (lambda a, b: ctx.apply_h(a, b, -0.4, dtype=tps.F64),
+                  lambda a, b: ctx.apply_prec(a, b, -0.4, dtype=tps.F64)):
+        apply(x, block)
+        for v in (0, nvec - 1):
+            apply(x[v:v + 1], one)
+            torch.cuda.synchronize()
+            assert torch.equal(block[v], one[0]), v
+    ctx.close()
