@@ -214,13 +214,13 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
     const int jl = 2 * c + (t & 1);
     const int j = j0 + 8 * gg + jl;
     if (!v || j >= g_.q) continue;
-    const unsigned er = (t & 2) ? eb : ea, fr = Fraw[gg][jl];
-    double val = 0.0;
+    double val;
     if constexpr (y_digits(KT) == 8) {
       int d[kUL];
 #pragma unroll
       for (int l = 0; l < kUL; ++l) d[l] = __float2int_rn(acc[gg][l][t]);
-      if (er && fr) val = level_sum(d, (int)er - 1022 + (int)fr - 1022, kWeights);
+      const unsigned er = (t & 2) ? eb : ea, fr = Fraw[gg][jl];
+      val = (er && fr) ? level_sum(d, (int)er - 1022 + (int)fr - 1022, kWeights) : 0.0;
     } else {  // (hi 2^32 + lo) 2^(E - 70): Horner sums in base 256 of levels 0-3 and 4-7
       long long hi = 0, lo = 0;
 #pragma unroll
@@ -231,7 +231,8 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
         else
           lo = lo * 256 + dl;
       }
-      if (er && fr) val = combine(hi, lo, (int)er - 1022 + (int)fr - 1022);
+      const unsigned er = (t & 2) ? eb : ea, fr = Fraw[gg][jl];
+      val = (er && fr) ? combine(hi, lo, (int)er - 1022 + (int)fr - 1022) : 0.0;
     }
     double *dst = Cs + (long long)j * g_.ldc + ((t & 2) ? rb : ra);
     *dst = g_.has_beta ? fma(g_.beta, *dst, val) : val;
