@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(64 * kGroups)
 k_linear_fwd(const float *__restrict__ X, int B, int in, const TW *__restrict__ W,
              const float *__restrict__ bias, int out, int act, float *__restrict__ Z,
              float *__restrict__ A) {
-  extern __shared__ float sh[];
+  extern __shared__ __align__(16) float sh[];
   const int r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
   const TileGemm<true, false, TW> g = {X, W, B, out, in, in, out};
   g.run(r0, c0, sh, nullptr);
@@ -170,7 +170,7 @@ k_linear_fwd(const float *__restrict__ X, int B, int in, const TW *__restrict__ 
 __global__ void __launch_bounds__(64 * kGroups)
 k_linear_wgrad(const float *__restrict__ X, int B, int in, const float *__restrict__ dZ, int out,
                float *__restrict__ dW, float *__restrict__ db) {
-  extern __shared__ float sh[];
+  extern __shared__ __align__(16) float sh[];
   __shared__ float bsum[kTile];
   const int i0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
   const TileGemm<false, false, float> g = {X, dZ, in, out, B, in, out};
@@ -187,7 +187,7 @@ k_linear_wgrad(const float *__restrict__ X, int B, int in, const float *__restri
 __global__ void __launch_bounds__(64 * kGroups)
 k_linear_xgrad(const float *__restrict__ dZ, int B, int out, const float *__restrict__ W, int in,
                const float *__restrict__ Zprev, float *__restrict__ dX) {
-  extern __shared__ float sh[];
+  extern __shared__ __align__(16) float sh[];
   const int r0 = blockIdx.y * kTile, i0 = blockIdx.x * kTile;
   const TileGemm<true, true, float> g = {dZ, W, B, in, out, out, out};
   g.run(r0, i0, sh, nullptr);
@@ -207,7 +207,7 @@ k_linear_xgrad(const float *__restrict__ dZ, int B, int out, const float *__rest
 __global__ void __launch_bounds__(256)
 k_cosine_loss(const float *__restrict__ out, int R, int px, int py, const float *__restrict__ T,
               float *__restrict__ G, double *__restrict__ loss, float inv_batch, int stage) {
-  extern __shared__ float sh[];
+  extern __shared__ __align__(16) float sh[];
   const int ld = py + stage;
   float *P = sh;  // px * ld, then dL/dP in its place
   __shared__ float red[3][8];

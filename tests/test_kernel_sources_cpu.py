@@ -1,7 +1,8 @@
-"""What a kernel may do before the one that it depends on has completed, read from its source.
+"""Rules of the kernels that no run can show, read from their sources.
 
-A kernel launched with the programmatic attribute may start before its predecessor in the stream
-has written its results, and only griddepcontrol.wait (pdl_wait) makes them visible.
+What a kernel may do before the one that it depends on has completed: launched with the
+programmatic attribute, it may start before its predecessor in the stream has written its results,
+and only griddepcontrol.wait (pdl_wait) makes them visible.  And the alignment of shared memory.
 """
 import glob
 import os
@@ -54,3 +55,13 @@ def test_dependents_start_after_the_tensor_memory_is_allocated(source, name):
     held = body.index("__syncthreads()", alloc)
     assert body.index("pdl_trigger()") > held
     assert "pdl_entry()" not in body
+
+
+def test_shared_memory_read_as_float4_is_declared_aligned():
+    # the layer products read their slabs, at the start of the dynamic array, as float4
+    with open(os.path.join(CSRC, "mlp.cu")) as f:
+        text = f.read()
+    assert "reinterpret_cast<const float4 *>" in text
+    declared = re.findall(r"extern __shared__([^;]*);", text)
+    assert len(declared) >= 4
+    assert all("__align__(16)" in d for d in declared), declared
