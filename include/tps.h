@@ -388,6 +388,16 @@ int tps_block_update_tc(tps_ctx *ctx, const double *A_dev, long long lda, int p,
                         const double *Y_dev, int ldy, int q, double beta, double *C_dev,
                         long long ldc, long long nrows, cudaStream_t stream);
 
+/* Self-test of the correction solve's Arnoldi pass (no solve shows its errors: the outer iteration
+ * absorbs them).  Per system s < batch, C_s -= A_s y_s (A_s: p <= 16 columns of nrows, lda apart;
+ * C_s: one column) and from the new C_s, in the same pass, G_s = A_s^T C_s (gram != 0) or
+ * G_s[0] = |C_s|^2.  FP32 products on the FP64 data, the norm in FP64.  Systems are bsa, bsy,
+ * bsc, bsg elements apart.  Device pointers. */
+int tps_selftest_arnoldi_pass(tps_ctx *ctx, const double *A_dev, long long lda, long long bsa,
+                              int p, const double *Y_dev, long long bsy, double *C_dev,
+                              long long bsc, long long nrows, int gram, double *G_dev,
+                              long long bsg, int batch, cudaStream_t stream);
+
 /* Orthonormalise the block T (b <= 32 columns) against the orthonormal block Q
  * (nq columns, may be 0) and within itself: two passes of block classical
  * Gram-Schmidt followed by Cholesky QR twice (Sec. 4.1, search-space expansion).

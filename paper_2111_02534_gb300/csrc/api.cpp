@@ -977,6 +977,21 @@ int tps_block_update_tc(tps_ctx *ctx, const double *A_dev, long long lda, int p,
   return TPS_OK;
 }
 
+int tps_selftest_arnoldi_pass(tps_ctx *ctx, const double *A_dev, long long lda, long long bsa,
+                              int p, const double *Y_dev, long long bsy, double *C_dev,
+                              long long bsc, long long nrows, int gram, double *G_dev,
+                              long long bsg, int batch, cudaStream_t stream) {
+  if (!ctx) return TPS_ERR_INVALID_ARG;
+  if (!update_then_supported(p) || batch < 1 || batch > 64 || nrows < 1 || lda < nrows ||
+      bsc < nrows || bsa < 0 || bsy < p || bsg < (gram ? p : 1) || !A_dev || !Y_dev || !C_dev ||
+      !G_dev)
+    return set_error(ctx, TPS_ERR_INVALID_ARG, "bad arnoldi_pass arguments");
+  launch_update_then(A_dev, lda, bsa, p, Y_dev, bsy, C_dev, bsc, nrows, gram != 0, G_dev, bsg,
+                     batch, ctx->gscr, stream);
+  TPS_CUDA_TRY(ctx, cudaGetLastError());
+  return TPS_OK;
+}
+
 int tps_small_eigh(tps_ctx *ctx, const double *G_dev, int m, int ldg, double *theta_dev,
                    double *Y_dev, int ldy, cudaStream_t stream) {
   if (!ctx) return TPS_ERR_INVALID_ARG;

@@ -110,6 +110,8 @@ _sig = {
                                    _vp, _ll, _ll, _vp]),
     "tps_block_update_tc": (C.c_int, [_vp, _vp, _ll, C.c_int, _vp, C.c_int, C.c_int, C.c_double,
                                       _vp, _ll, _ll, _vp]),
+    "tps_selftest_arnoldi_pass": (C.c_int, [_vp, _vp, _ll, _ll, C.c_int, _vp, _ll, _vp, _ll, _ll,
+                                            C.c_int, _vp, _ll, C.c_int, _vp]),
     "tps_orthonormalize": (C.c_int, [_vp, _vp, _ll, C.c_int, _vp, _ll, C.c_int, _ll, _ip, _vp]),
     "tps_small_eigh": (C.c_int, [_vp, _vp, C.c_int, C.c_int, _vp, _vp, C.c_int, _vp]),
     "tps_correction": (C.c_int, [_vp, _vp, C.c_int, _vp, _vp, C.c_int, C.c_int, C.c_int,
