@@ -95,7 +95,7 @@ __device__ __forceinline__ bool halving_writer(int lane) {  // one lane per valu
 // The sum of acc over the threads of all nchunk CTAs that share `partial` and `count`, chunk c's
 // share first reduced in its CTA.  True in the last CTA to arrive, whose tot[0 .. V) then holds
 // the sums, added in an order that does not depend on scheduling; it re-arms the counter for
-// the next call on this stream.
+// the next call on this stream.  One chunk needs neither memory nor ticket.
 template <typename T, int V>
 __device__ __forceinline__ bool chunk_sums(T (&acc)[V], double *partial, unsigned *count, int c,
                                            int nchunk, double (&tot)[GT]) {
@@ -108,10 +108,15 @@ __device__ __forceinline__ bool chunk_sums(T (&acc)[V], double *partial, unsigne
   if (threadIdx.x < V) {
     T v = T(0);
     for (int w = 0; w < GT / 32; ++w) v += red[w][threadIdx.x];
-    partial[c * V + threadIdx.x] = (double)v;
-    __threadfence();  // this chunk's sums are visible before the ticket is taken
+    if (nchunk == 1) {
+      tot[threadIdx.x] = (double)v;
+    } else {
+      partial[c * V + threadIdx.x] = (double)v;
+      __threadfence();  // this chunk's sums are visible before the ticket is taken
+    }
   }
   __syncthreads();
+  if (nchunk == 1) return true;
   if (threadIdx.x == 0) ticket = atomicAdd(count, 1u);
   __syncthreads();
   if (ticket != (unsigned)(nchunk - 1)) return false;
@@ -139,8 +144,12 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
        const double *__restrict__ B, long long ldb, long long bsb, int q, long long nrows,
        int nchunk, double *__restrict__ partial, unsigned *__restrict__ count,
        double *__restrict__ G, int ldg, long long bsg, int trans, const int *__restrict__ need) {
-  pdl_entry();
   constexpr int V = BP * BQ;
+  constexpr bool kFma = sizeof(T) == 8 && V == 16 && BQ > 1;
+  if constexpr (kFma)
+    pdl_wait();
+  else
+    pdl_entry();
   if (need && *need == 0) return;  // conditional product (decided on the device)
   const int c = blockIdx.x, s = blockIdx.y, pb = blockIdx.z;
   const int qb = (q + BQ - 1) / BQ;
@@ -148,15 +157,27 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
   const int i0 = (pb / qb) * BP, j0 = (pb % qb) * BQ;
   const double *As = A + s * bsa;
   const double *Bs = B + s * bsb;
-  // the chunks' rows are interleaved, so that the CTAs read neighbouring addresses of the
-  // p + q columns at any time and few pages of memory are in use at once
-  const long long step = (long long)nchunk * GT;
+  // Where memory is the bound, the chunks' rows are interleaved, so that the CTAs read neighbouring
+  // addresses of the p + q columns at any time and few pages of memory are in use at once.
+  //
+  // FP64 tiles of 16 values from several columns are bound by the FMA pipe.  Their chunks are runs
+  // of rows: a constant distance of the two rows of an iteration lets the compiler keep the loads of
+  // both in flight (112 registers instead of 80; p = 64, q = 2, 1 M rows 222 us instead of 232).
+  // And they start their dependents after their FMAs: the CTAs of a dependent that wait on the SMs
+  // from the start are packed unevenly beside this kernel's, and then two share one SM's pipe while
+  // others idle.  Back to back, runs and late against interleaved and early: 131,584 rows, p = q = 8
+  // 21.6 and 29.9 us; 10,000 rows 16 x 8 10.0 and 19.2, 8 x 8 9.9 and 10.5; 5.3 M rows 16 x 8 1116
+  // and 1134.  Narrow tiles lose by both (p = 8, q = 1, 5.3 M rows 83 us, 120 in runs).
+  const long long rows_per = (nrows + nchunk - 1) / nchunk;
+  const long long r0 = (long long)c * (kFma ? rows_per : GT);
+  const long long r1 = kFma && r0 + rows_per < nrows ? r0 + rows_per : nrows;
+  const long long step = kFma ? GT : (long long)nchunk * GT;
   T acc[V];
 #pragma unroll
   for (int k = 0; k < V; ++k) acc[k] = T(0);
   // two rows per iteration: all of their loads are issued before the first FMA waits
-  long long r = (long long)c * GT + threadIdx.x;
-  for (; r + step < nrows; r += 2 * step) {
+  long long r = r0 + threadIdx.x;
+  for (; r + step < r1; r += 2 * step) {
     T a[2][BP], b[2][BQ];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -174,7 +195,7 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
 #pragma unroll
         for (int j = 0; j < BQ; ++j) acc[i * BQ + j] = fma(a[h][i], b[h][j], acc[i * BQ + j]);
   }
-  if (r < nrows) {
+  if (r < r1) {
     T a[BP], b[BQ];
 #pragma unroll
     for (int i = 0; i < BP; ++i)
@@ -187,6 +208,7 @@ k_gram(const double *__restrict__ A, long long lda, long long bsa, int p,
 #pragma unroll
       for (int j = 0; j < BQ; ++j) acc[i * BQ + j] = fma(a[i], b[j], acc[i * BQ + j]);
   }
+  if constexpr (kFma) pdl_trigger();
   __shared__ double tot[GT];
   const long long blk = (long long)s * npb + pb;
   if (!chunk_sums<T, V>(acc, partial + blk * nchunk * V, count + blk, c, nchunk, tot)) return;

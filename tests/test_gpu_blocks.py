@@ -288,3 +288,21 @@ def test_correction_matches_textbook_gmres():
         x, _ = blocks.gmres(A, b, steps)
         assert np.linalg.norm(got[i] - x) <= 1e-9 * np.linalg.norm(x)
         assert abs(Qt.T @ got[i]).max() <= 1e-10 * np.linalg.norm(got[i])
+
+
+@pytest.mark.parametrize("nrows", [1, 255, 257, 1024, 1025, 2049, 33333, 400003])
+@pytest.mark.parametrize("p,q", [(8, 2), (9, 2), (3, 3), (8, 3), (5, 8), (13, 8)])
+def test_gram_fp64_chunks(ctx, nrows, p, q):
+    # the tiles of 16 values in several columns: one chunk, two, a last chunk without rows, odd
+    # numbers of rows per thread.  At most 64 roundings follow one another: the rows of a thread (21
+    # here), five steps in the warp, eight warps, the chunks
+    g = torch.Generator(device="cuda").manual_seed(nrows)
+    A = torch.randn(p, nrows, generator=g, dtype=torch.float64, device="cuda")
+    B = torch.randn(q, nrows, generator=g, dtype=torch.float64, device="cuda")
+    G = torch.full((3, q, p), np.nan, dtype=torch.float64, device="cuda")
+    for i in range(3):  # one behind the other: each waits for the scratch of the one before
+        ctx.gram(A, p, B, q, nrows, G[i])
+    a, b = host(A), host(B)
+    got = host(G[0]).T
+    assert np.all(np.abs(got - _exact_gram(a, b)) <= 64 * 2.0 ** -53 * (np.abs(a) @ np.abs(b).T))
+    assert torch.equal(G[0], G[1]) and torch.equal(G[0], G[2])
