@@ -178,8 +178,9 @@ __device__ __forceinline__ void digit_pairs(uint64_t u0, uint64_t u1, uint32_t (
   }
 }
 
-// Digit j of the 62-bit integer round(x 2^(62 - E)), E = raw_max - 1022, in eight digits.
-__device__ __forceinline__ int digit62(double x, unsigned raw_max, int j) {
+// round(x 2^(62 - E)) + 128 (1 + 2^8 + .. + 2^56), E = raw_max - 1022: its bytes are the eight
+// digits of the 62-bit integer plus 128.
+__device__ __forceinline__ unsigned long long biased62(double x, unsigned raw_max) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int raw = (int)((b >> 52) & 0x7FF);
   long long q = 0;
@@ -192,8 +193,13 @@ __device__ __forceinline__ int digit62(double x, unsigned raw_max, int j) {
       q = (mant + (1LL << (-sh - 1))) >> (-sh);
     if (b >> 63) q = -q;
   }
-  const unsigned long long u = (unsigned long long)q + 0x8080808080808080ULL;
+  return (unsigned long long)q + 0x8080808080808080ULL;
+}
+__device__ __forceinline__ int digit(unsigned long long u, int j) {
   return (int)((u >> (8 * (7 - j))) & 0xFF) - 128;
+}
+__device__ __forceinline__ int digit62(double x, unsigned raw_max, int j) {
+  return digit(biased62(x, raw_max), j);
 }
 
 // sum_l d_l 2^(104 - 8 l) 2^(E - 117) rounded to FP64: the levels of seven digits of A (scale

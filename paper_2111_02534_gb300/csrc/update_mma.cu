@@ -15,10 +15,11 @@
 //    integer below 2^23.6 for p <= 64);
 //  * the levels are combined in two int64 Horner sums (levels 0-3 and 4-7) and rounded once to
 //    FP64 by integer arithmetic; for p <= 16 they add up in one 64-bit integer, which the FP64
-//    pipe rounds (p = 16, q = 3, 5.3 M rows: 438 -> 360 us).
-// The dropped levels l >= 8 weigh at most 131072 p 2^(E_r + F_j - 78) < p 2^-61 2^(E_r +
-// F_j) per entry, and the truncation of the operands to 55 bits 2^-55 of the row maximum:
-// the result has the accuracy of an FP64 product, 2^-53 max_k |A[r][k]| sum_k |alpha Y[k][j]|
+//    pipe rounds (p = 16: q = 3, 5.3 M rows 476 -> 357 us; q = 8, 131,584 rows 16.4 -> 13.7).
+// The dropped levels l >= 8 weigh at most 2^17 p 2^(E_r + F_j - 78) = p 2^-61 2^(E_r + F_j) per
+// entry (l = 8; the rest a hundredth of it), twice that for p <= 16, whose digits of alpha Y weigh twice as much,
+// where also level 7 is rounded to 2^-62 2^(E_r + F_j); the truncation of the operands to 55 bits
+// 2^-55 of the row maximum: the result has the accuracy of an FP64 product, 2^-53 max_k |A[r][k]| sum_k |alpha Y[k][j]|
 // per entry (row-wise, not element-wise).
 //
 // The MMA is the warp-level mma.sync m16n8k16 (BF16 in, FP32 out): the output is only
@@ -38,6 +39,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "ozaki_tc.cuh"
 #include "split_digits.cuh"
@@ -206,24 +208,51 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
     }
   }
   // combine the levels
+  if constexpr (y_digits(KT) == 8) {
+    // the old values are loaded together, ahead of the sums they are added to: one by one behind
+    // level_sum's branch they cost 5 us of 19.5 (p = 16, q = 8, 131,584 rows)
+    auto finish = [&](auto with_old) {
+      constexpr bool kOld = decltype(with_old)::value;
 #pragma unroll
-  for (int gg = 0; gg < NG; ++gg)
+      for (int gg = 0; gg < NG; ++gg) {
+        double old[4];
+        bool in[4];
 #pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const bool v = (t & 2) ? vb : va;
-    const int jl = 2 * c + (t & 1);
-    const int j = j0 + 8 * gg + jl;
-    if (!v || j >= g_.q) continue;
-    double val;
-    if constexpr (y_digits(KT) == 8) {
-      int d[kUL];
+        for (int t = 0; t < 4; ++t) {
+          const int j = j0 + 8 * gg + 2 * c + (t & 1);
+          in[t] = ((t & 2) ? vb : va) && j < g_.q;
+          if (kOld && in[t]) old[t] = Cs[(long long)j * g_.ldc + ((t & 2) ? rb : ra)];
+        }
 #pragma unroll
-      for (int l = 0; l < kUL; ++l) d[l] = __float2int_rn(acc[gg][l][t]);
-      const unsigned er = (t & 2) ? eb : ea, fr = Fraw[gg][jl];
-      val = (er && fr) ? level_sum(d, (int)er - 1022 + (int)fr - 1022, kWeights) : 0.0;
-    } else {  // (hi 2^32 + lo) 2^(E - 70): Horner sums in base 256 of levels 0-3 and 4-7
-      long long hi = 0, lo = 0;
+        for (int t = 0; t < 4; ++t) {
+          if (!in[t]) continue;
+          const int jl = 2 * c + (t & 1);
+          int d[kUL];
 #pragma unroll
+          for (int l = 0; l < kUL; ++l) d[l] = __float2int_rn(acc[gg][l][t]);
+          const unsigned er = (t & 2) ? eb : ea, fr = Fraw[gg][jl];
+          const double val =
+              (er && fr) ? level_sum(d, (int)er - 1022 + (int)fr - 1022, kWeights) : 0.0;
+          Cs[(long long)(j0 + 8 * gg + jl) * g_.ldc + ((t & 2) ? rb : ra)] =
+              kOld ? fma(g_.beta, old[t], val) : val;
+        }
+      }
+    };
+    if (g_.has_beta)
+      finish(std::true_type{});
+    else
+      finish(std::false_type{});
+  } else {
+#pragma unroll
+    for (int gg = 0; gg < NG; ++gg)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const bool v = (t & 2) ? vb : va;
+      const int jl = 2 * c + (t & 1);
+      const int j = j0 + 8 * gg + jl;
+      if (!v || j >= g_.q) continue;
+      long long hi = 0, lo = 0;  // (hi 2^32 + lo) 2^(E - 70): Horner sums in base 256 of levels
+#pragma unroll                 // 0-3 and 4-7
       for (int l = 0; l < kUL; ++l) {
         const long long dl = (long long)__float2int_rn(acc[gg][l][t]);
         if (l < kUL / 2)
@@ -232,10 +261,10 @@ __device__ __forceinline__ void block16(const UpdArgs &g_, const double *As, Str
           lo = lo * 256 + dl;
       }
       const unsigned er = (t & 2) ? eb : ea, fr = Fraw[gg][jl];
-      val = (er && fr) ? combine(hi, lo, (int)er - 1022 + (int)fr - 1022) : 0.0;
+      const double val = (er && fr) ? combine(hi, lo, (int)er - 1022 + (int)fr - 1022) : 0.0;
+      double *dst = Cs + (long long)j * g_.ldc + ((t & 2) ? rb : ra);
+      *dst = g_.has_beta ? fma(g_.beta, *dst, val) : val;
     }
-    double *dst = Cs + (long long)j * g_.ldc + ((t & 2) ? rb : ra);
-    *dst = g_.has_beta ? fma(g_.beta, *dst, val) : val;
   }
 }
 
@@ -251,11 +280,7 @@ __device__ __forceinline__ void y_fragments(const UpdArgs &g_, const double *Ys,
     const int jl = t >> 4, k0 = t & 15, j = j0 + jl;
     unsigned m = 0;
     if constexpr (YS == 8) {
-      double sum = 0.0;
-      if (j < g_.q)
-#pragma unroll
-        for (int k = k0; k < 64; k += 16)
-          if (k < g_.p) sum += fabs(g_.alpha * Ys[(long long)j * g_.ldy + k]);
+      double sum = j < g_.q && k0 < g_.p ? fabs(g_.alpha * Ys[(long long)j * g_.ldy + k0]) : 0.0;
 #pragma unroll
       for (int o = 1; o < 16; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       m = raw_exp(sum);
@@ -270,7 +295,7 @@ __device__ __forceinline__ void y_fragments(const UpdArgs &g_, const double *Ys,
     if (k0 == 0) Fraw[jl] = m;
   }
   asm volatile("bar.sync 1, %0;" ::"r"(kCons) : "memory");
-  if (t < 32 * kUKT) {
+  if (t < 32 * (YS == 8 ? 1 : kUKT)) {  // eight digits go with one k tile
     const int kt = t >> 5, lane = t & 31, g = lane >> 2, c = lane & 3;
     const int j = j0 + g;
     float dv[4][YS];
@@ -279,8 +304,9 @@ __device__ __forceinline__ void y_fragments(const UpdArgs &g_, const double *Ys,
       const int k = 16 * kt + 2 * c + (e & 1) + 8 * (e >> 1);
       const double y = (j < g_.q && k < g_.p) ? g_.alpha * Ys[(long long)j * g_.ldy + k] : 0.0;
       if constexpr (YS == 8) {
+        const unsigned long long u = biased62(y, Fraw[g]);
 #pragma unroll
-        for (int i = 0; i < YS; ++i) dv[e][i] = (float)digit62(y, Fraw[g], i);
+        for (int i = 0; i < YS; ++i) dv[e][i] = (float)digit(u, i);
       } else {
         digits7(y, Fraw[g], dv[e]);
       }

@@ -306,3 +306,25 @@ def test_gram_fp64_chunks(ctx, nrows, p, q):
     got = host(G[0]).T
     assert np.all(np.abs(got - _exact_gram(a, b)) <= 64 * 2.0 ** -53 * (np.abs(a) @ np.abs(b).T))
     assert torch.equal(G[0], G[1]) and torch.equal(G[0], G[2])
+
+
+@pytest.mark.parametrize("nrows", [1, 17, 127, 128, 130, 10001, 131590])
+@pytest.mark.parametrize("p,q", [(1, 1), (8, 8), (9, 5), (16, 3), (13, 16), (16, 24), (16, 30)])
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+def test_block_update_tc_narrow(ctx, nrows, p, q, beta):
+    # at most 16 columns, whose levels add up in one integer, on rows and columns of very different
+    # size: the scheme's bound as above, the dropped digit pairs p 2^-60 of the row's exponent
+    # (twice its maximum) times that of the column's absolute sum (twice it), the last FMA's rounding
+    from paper_2111_02534_gb300 import tps
+    rng = np.random.default_rng(nrows + p)
+    A = rng.standard_normal((p, nrows)) * 10.0 ** rng.uniform(-12, 12, nrows)[None, :]
+    A[:, ::97] = 0.0
+    Y = rng.standard_normal((p, q)) * 10.0 ** rng.uniform(-8, 8, q)[None, :]
+    C0 = rng.standard_normal((q, nrows))
+    Cd = dev(C0)
+    ctx.block_update(dev(A), p, dev(Y.T.copy()), q, beta, Cd, nrows, ldy=p, dtype=tps.F64_TC)
+    ref = (beta * C0.astype(np.longdouble) + Y.T.astype(np.longdouble) @ A.astype(np.longdouble))
+    size = np.outer(np.abs(Y).sum(axis=0), np.abs(A).max(axis=0))
+    bound = (4 * 2.0 ** -53 + 4 * p * 2.0 ** -60) * size + 2.0 ** -52 * np.abs(C0)
+    assert np.all(np.abs(host(Cd) - ref) <= bound)
+    assert np.all(host(Cd)[:, ::97] == beta * C0[:, ::97])
