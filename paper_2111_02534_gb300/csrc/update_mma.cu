@@ -17,10 +17,10 @@
 //    FP64 by integer arithmetic; for p <= 16 they add up in one 64-bit integer, which the FP64
 //    pipe rounds (p = 16: q = 3, 5.3 M rows 476 -> 357 us; q = 8, 131,584 rows 16.4 -> 13.7).
 // The dropped levels l >= 8 weigh at most 2^17 p 2^(E_r + F_j - 78) = p 2^-61 2^(E_r + F_j) per
-// entry (l = 8; the rest a hundredth of it), twice that for p <= 16, whose digits of alpha Y weigh twice as much,
-// where also level 7 is rounded to 2^-62 2^(E_r + F_j); the truncation of the operands to 55 bits
-// 2^-55 of the row maximum: the result has the accuracy of an FP64 product, 2^-53 max_k |A[r][k]| sum_k |alpha Y[k][j]|
-// per entry (row-wise, not element-wise).
+// entry (l = 8; the rest a hundredth of it), twice that for p <= 16, whose digits of alpha Y weigh
+// twice as much, where also level 7 is rounded to 2^-62 2^(E_r + F_j); the truncation of the
+// operands to 55 bits 2^-55 of the row maximum: the result has the accuracy of an FP64 product,
+// 2^-53 max_k |A[r][k]| sum_k |alpha Y[k][j]| per entry (row-wise, not element-wise).
 //
 // The MMA is the warp-level mma.sync m16n8k16 (BF16 in, FP32 out): the output is only
 // q <= 8 columns wide, and a tcgen05.mma costs its issuing thread about 45 cycles
