@@ -67,7 +67,7 @@ struct TileGemm {
     }
   }
   __device__ __forceinline__ void load(int t, int m0, int n0, int k0, float (&a)[8],
-                                       float (&b)[8]) const {
+                                       TB (&b)[8]) const {
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       int r, k;
@@ -77,9 +77,9 @@ struct TileGemm {
                  : 0.f;
       place(BK, t, e, r, k);
       b[e] = (n0 + r < N && k0 + k < K)
-                 ? (float)B[BK ? (long long)(n0 + r) * ldb + k0 + k
-                               : (long long)(k0 + k) * ldb + n0 + r]
-                 : 0.f;
+                 ? B[BK ? (long long)(n0 + r) * ldb + k0 + k
+                        : (long long)(k0 + k) * ldb + n0 + r]
+                 : TB(0.f);
     }
   }
   // The tile's sums in sh[m][n] (32 x 32) for all threads; bsum (nullable): sum_k B(k, n) of the
@@ -89,7 +89,8 @@ struct TileGemm {
     float(*as)[kLd] = reinterpret_cast<float(*)[kLd]>(sh + g * 2 * kSlab * kLd);
     float(*bs)[kLd] = as + kSlab;
     float acc[4][4] = {}, bacc[4] = {};
-    float a[8], b[8];
+    float a[8];
+    TB b[8];  // converted when stored: a conversion here would wait for the loads
     load(t, m0, n0, g * kSlab, a, b);
     for (int k0 = g * kSlab; k0 < K; k0 += kGroups * kSlab) {
 #pragma unroll
@@ -98,7 +99,7 @@ struct TileGemm {
         place(AK, t, e, r, k);
         as[k][r] = a[e];
         place(BK, t, e, r, k);
-        bs[k][r] = b[e];
+        bs[k][r] = (float)b[e];
       }
       asm volatile("bar.sync %0, 64;" ::"r"(1 + g) : "memory");
       load(t, m0, n0, k0 + kGroups * kSlab, a, b);  // zeros past the end
