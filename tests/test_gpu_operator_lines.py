@@ -106,3 +106,32 @@ def test_blocks_of_more_vectors_than_a_launch_takes(n, nvec):
             ctx.device_status()
             assert torch.equal(out[v], one[0]), v
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [(64, 66), (60, 130), (12, 12, 18, 18), (6, 6, 48, 48)])
+@pytest.mark.parametrize("k", [-1015, -1000, -960, -940, 870, 900, 930, 1000])
+def test_results_near_the_ends_of_the_range(n, k):
+    # the recombination scales by exponent arithmetic, near the ends of FP64's range in two factors:
+    # a wave function times 2^k against the plain one, whose sums are the same integers.  The mode
+    # products count subnormals as zero; the potential term takes them as they are
+    require_gpu()
+    from paper_2111_02534_gb300 import tps
+    L = (9.0,) * len(n)
+    ctx = (make_ctx_1d if len(n) == 2 else make_ctx_2d)(20.0, 1.0, n, L, 1.0, 1.0)
+    N, hn = ctx.info()
+    assert hn < 2.0 ** 12
+    V = -np.random.default_rng(5).random(N)
+    ctx.set_potential(V)
+    psi = _random(2, N, 11)
+    ref, out = torch.empty_like(psi), torch.empty_like(psi)
+    big = psi * 2.0 ** k
+    kept = torch.where(big.abs() >= 2.0 ** -1022, psi, 0.0)
+    ctx.apply_h(kept, ref, -0.3, dtype=tps.F64_TC)
+    ref += (torch.from_numpy(V).cuda() + 0.3) * (psi - kept)
+    ctx.apply_h(big, out, -0.3, dtype=tps.F64_TC)
+    ctx.device_status()
+    # below 2^-1022 a result has 2^-1074 left, 2^-59 of the scale here
+    bound = 1e-14 * hn * float(psi.abs().max())
+    assert bool(out.isfinite().all())
+    assert bool(((out * 2.0 ** -k - ref).abs() <= bound).all())
+    ctx.close()
