@@ -753,7 +753,8 @@ int tps_ws_loss_grad(tps_ws *ws, const float *X_dev, const float *T_dev, int B, 
                                   cudaMemcpyDeviceToDevice, stream));
   forward(ws, B, false, stream);
   // loss and dL/d(output) into dZa
-  const size_t plain = sizeof(float) * 2 * ws->px * ws->py;  // as many modes as before fit
+  // the sizes accepted are those of two px x py matrices in 48 KB, whichever form runs
+  const size_t plain = sizeof(float) * 2 * ws->px * ws->py;
   const size_t staged = sizeof(float) * ((size_t)ws->px * (ws->py + 1) + ws->dims[kLayers]);
   const int stage = staged <= (48u << 10) && plain <= (48u << 10) ? 1 : 0;
   tps::count_launch();

@@ -13,12 +13,16 @@
 // 146 points) for base-256 digits, 36 digit products instead of the 54 that base 64 needs for
 // 512 points, so that of the tensor work of the dense product a sixth is left.
 //
-// Everything but the last rounding is exact integer arithmetic: a line of psi is scaled by a
-// power of two and rounded to 62 - log2|G| bits, the sums F_b are taken in 64-bit integers and
-// cut into eight base-256 digits, the entries of |G| B_b likewise (62 bits of the row's absolute
-// sum).  The eight levels of digit products (ozaki_tc.cu) are added to one 64-bit integer per
-// Z_b[r], with a common unit for all blocks, and the sums over b are again exact.  A product is
-// rounded once, as in the dense scheme, from operands that keep 60 bits instead of 54.
+// The arithmetic between the rounding of the operands and that of the result is on integers: a
+// line of psi is scaled by a power of two and rounded to 62 - log2|G| bits, the sums F_b are taken
+// in 64-bit integers and cut into eight base-256 digits, the entries of |G| B_b likewise (62 bits
+// of the row's absolute sum).  The eight levels of digit products (ozaki_tc.cu) are exact; they are
+// added to one 64-bit integer per Z_b[r], with a common unit u for all blocks (2^-62 of the line's
+// scale times the row's), level 7 rounded to u, and the sums over b are again exact.  Left out are
+// the digit pairs with i + j >= 8: of a block of 146 points at most 7 2^14 146 2^-14 = 1022 u, about
+// 11 u as a root mean square, twice and four times that for a result of four blocks (2^-57 and, at
+// most, 2^-50 of the scales; an FP64 product of 512 terms is bounded by 2^-44 of them).  A product
+// is rounded once, as in the dense scheme, whose psi keeps 54 bits.
 //
 // Three kernels:
 //   k_fold_split    reads 16 lines (rows for y, columns for x) into shared memory, takes their
@@ -32,7 +36,7 @@
 //   k_fold_combine  a thread per pair of representatives (r_x, r_y) and image of r_x: unfolds
 //                   both modes, adds the potential term and writes the |G_y| outputs.
 //
-// Measured, 8 vectors at 512 x 512: 119 us, 476 by the dense base-64 products.
+// Measured, 8 vectors at 512 x 512: 102 us, 476 by the dense base-64 products.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 

@@ -4,14 +4,14 @@
 //
 //   out[m][j] (+)= sum_i psi[m][i] K[j][i],   m a fiber of the mode, i, j its points
 //
-// What bounds it: the integer pipe.  An element costs about 35 integer and packed FP16
-// instructions to cut into digits and an output about 45 to put together from its eight
-// levels; the ALU (16 lanes per cycle and scheduler) is 59 % busy, issue 62 %, and the 24 bytes
-// per element and mode that have to move (psi read, out read and written) take 0.62 of the time
-// at the copy rate.  (A split kernel that writes the digits to memory and a product kernel that
-// reads them back move 54 bytes.)  Measured at 48^4 for 3 vectors: 100 us for each of y1, x2 and
-// x1, 115 for y2, 63 for the potential term; a whole apply of 8 vectors 1.18 ms, 3.62 with the
-// split and product kernels.
+// What bounds it: the integer pipe.  An output costs about 124 instructions of a lane in all (118
+// where it is stored), most of them to cut an element into digits and to put an output together
+// from its eight levels; the ALU (16 lanes per cycle and scheduler) is 56 % busy, issue 61 %, and
+// the 24 bytes per element and mode that have to move (psi read, out read and written) take 0.6 of
+// the time at the copy rate.  (A split kernel that writes the digits to memory and a product kernel
+// that reads them back move 54 bytes.)  Measured at 48^4 for 3 vectors: 94 us for each of y1, x2 and
+// x1, 107 for y2, 64 for the potential term; a whole apply of 8 vectors 1.13 ms, 3.63 with the split
+// and product kernels.
 //
 // One CTA per SM works through tiles of 128 fibers, every stage of several tiles in flight
 // (warps for a mode of 33 to 48 points):
@@ -21,8 +21,7 @@
 //   warps 12-27  copy the operator's image, then drain the accumulators, recombine the levels
 //                and store;
 //   warp 28      issues the MMAs.
-// (Eight producer and eight epilogue warps, with twice the registers: 115 us per mode instead
-// of 100.)
+// (Eight producer and eight epilogue warps, with twice the registers, took 15 % more.)
 // The output columns are taken 16 at a time, eight levels x 16 columns = 128 TMEM columns, so
 // that four of these sub-tiles fit in tensor memory and the epilogue of one runs under the MMAs
 // of the next.  A narrow MMA costs ~45 cycles whatever its width (measured), and a product of

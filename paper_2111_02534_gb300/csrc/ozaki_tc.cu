@@ -1254,7 +1254,8 @@ cudaError_t ensure_tc_operator(const DevOperator &op, cudaStream_t s) {
 
 // 2D H-apply (Eq. tensor_op2D): the four mode products one after the other, each as
 // C[m][j] = sum_i Psi[fiber m][i] K_k[j][i] over the fibers of mode k (A = fiber slices,
-// B = K_k slices); the y2 product stores its tiles with the (V - theta) Psi term, the
+// B = K_k slices), the fused form taking the fibers themselves; the y2 product stores its tiles,
+// the dense one with the (V - theta) Psi term, which follows by itself after the fused one; the
 // other three add theirs (one CTA per output tile in each launch, so the sum is
 // deterministic).
 cudaError_t launch_apply_h_tc_2d(const DevOperator &op, const double *psi, double *out,
@@ -1357,7 +1358,8 @@ cudaError_t launch_apply_h_tc(const DevOperator &op, const double *psi, double *
   TcOperator &t = *op.tc;
   // modes that fold into blocks of at most 146 points (periodic grids of 4 k points up to 580,
   // of 2 k points up to 290, their sectors, anything up to 146): 8 vectors at 512 x 512 take
-  // 119 us that way and 476 us by the dense products below
+  // 102 us that way and 476 us by the dense products below.  What does not fold that far (periodic
+  // grids of 2 k points from 294 on, of 4 k above 580, and with them the other mode) stays dense
   if (t.fold) return ozf::apply(*t.fold, op, psi, out, nvec, theta_dev, theta, s);
   const int nx = t.nx, ny = t.ny, So = t.So, Sp = t.Sp;
   for (int v0 = 0; v0 < nvec; v0 += t.chunk) {
